@@ -70,27 +70,27 @@ static int arg_fail(const std::string &what) {
 // random sputtering matrix x physics variant, one storage type
 template <int ST, bool RS>
 static cudaError_t launch_step_phys(const StepArgs &a, int layout, int ns, int parity, cudaStream_t st,
-                                   const cudaEvent_t *ev) {
+                                   const cudaEvent_t *ev, bool first, bool last) {
   switch (a.phys) {
-    case kPhysBary: return launch_step_st<ST, RS, kPhysBary>(a, layout, ns, parity, st, ev);
-    case kPhysChannel: return launch_step_st<ST, RS, kPhysChannel>(a, layout, ns, parity, st, ev);
-    default: return launch_step_st<ST, RS, kPhysCarrier>(a, layout, ns, parity, st, ev);
+    case kPhysBary: return launch_step_st<ST, RS, kPhysBary>(a, layout, ns, parity, st, ev, first, last);
+    case kPhysChannel: return launch_step_st<ST, RS, kPhysChannel>(a, layout, ns, parity, st, ev, first, last);
+    default: return launch_step_st<ST, RS, kPhysCarrier>(a, layout, ns, parity, st, ev, first, last);
   }
 }
 
 template <int ST>
 static cudaError_t launch_step_modes(const StepArgs &a, int layout, int ns, int parity, cudaStream_t st,
-                                     const cudaEvent_t *ev) {
-  return a.rs ? launch_step_phys<ST, true>(a, layout, ns, parity, st, ev)
-              : launch_step_phys<ST, false>(a, layout, ns, parity, st, ev);
+                                     const cudaEvent_t *ev, bool first, bool last) {
+  return a.rs ? launch_step_phys<ST, true>(a, layout, ns, parity, st, ev, first, last)
+              : launch_step_phys<ST, false>(a, layout, ns, parity, st, ev, first, last);
 }
 
 cudaError_t launch_step(const StepArgs &a, int storage, int layout, int ns, int parity, cudaStream_t st,
-                        const cudaEvent_t *ev) {
+                        const cudaEvent_t *ev, bool first, bool last) {
   switch (storage) {
-    case LBM_FP32: return launch_step_modes<LBM_FP32>(a, layout, ns, parity, st, ev);
-    case LBM_FP16_DEV: return launch_step_modes<LBM_FP16_DEV>(a, layout, ns, parity, st, ev);
-    default: return launch_step_modes<LBM_BF16_DEV>(a, layout, ns, parity, st, ev);
+    case LBM_FP32: return launch_step_modes<LBM_FP32>(a, layout, ns, parity, st, ev, first, last);
+    case LBM_FP16_DEV: return launch_step_modes<LBM_FP16_DEV>(a, layout, ns, parity, st, ev, first, last);
+    default: return launch_step_modes<LBM_BF16_DEV>(a, layout, ns, parity, st, ev, first, last);
   }
 }
 
@@ -118,27 +118,28 @@ static cudaError_t launch_batch(const BatchLaunch &p, int storage, int layout, i
 }
 
 template <int ST, bool RS>
-static cudaError_t launch_batch_split_phys(const BatchLaunch &p, int layout, int ns, int det, cudaStream_t st) {
+static cudaError_t launch_batch_split_phys(const BatchLaunch &p, int layout, int ns, int det, cudaStream_t st,
+                                           bool first, bool last) {
   switch (p.v[0][0].phys) {
-    case kPhysBary: return launch_batch_split_st<ST, RS, kPhysBary>(p, layout, ns, det, st);
-    case kPhysChannel: return launch_batch_split_st<ST, RS, kPhysChannel>(p, layout, ns, det, st);
-    default: return launch_batch_split_st<ST, RS, kPhysCarrier>(p, layout, ns, det, st);
+    case kPhysBary: return launch_batch_split_st<ST, RS, kPhysBary>(p, layout, ns, det, st, first, last);
+    case kPhysChannel: return launch_batch_split_st<ST, RS, kPhysChannel>(p, layout, ns, det, st, first, last);
+    default: return launch_batch_split_st<ST, RS, kPhysCarrier>(p, layout, ns, det, st, first, last);
   }
 }
 
 static cudaError_t launch_batch_split(const BatchLaunch &p, int storage, int layout, int ns, int det,
-                                      cudaStream_t st) {
+                                      cudaStream_t st, bool first, bool last) {
   const bool rs = p.v[0][0].rs != 0;
   switch (storage) {
     case LBM_FP32:
-      return rs ? launch_batch_split_phys<LBM_FP32, true>(p, layout, ns, det, st)
-                : launch_batch_split_phys<LBM_FP32, false>(p, layout, ns, det, st);
+      return rs ? launch_batch_split_phys<LBM_FP32, true>(p, layout, ns, det, st, first, last)
+                : launch_batch_split_phys<LBM_FP32, false>(p, layout, ns, det, st, first, last);
     case LBM_FP16_DEV:
-      return rs ? launch_batch_split_phys<LBM_FP16_DEV, true>(p, layout, ns, det, st)
-                : launch_batch_split_phys<LBM_FP16_DEV, false>(p, layout, ns, det, st);
+      return rs ? launch_batch_split_phys<LBM_FP16_DEV, true>(p, layout, ns, det, st, first, last)
+                : launch_batch_split_phys<LBM_FP16_DEV, false>(p, layout, ns, det, st, first, last);
     default:
-      return rs ? launch_batch_split_phys<LBM_BF16_DEV, true>(p, layout, ns, det, st)
-                : launch_batch_split_phys<LBM_BF16_DEV, false>(p, layout, ns, det, st);
+      return rs ? launch_batch_split_phys<LBM_BF16_DEV, true>(p, layout, ns, det, st, first, last)
+                : launch_batch_split_phys<LBM_BF16_DEV, false>(p, layout, ns, det, st, first, last);
   }
 }
 
@@ -964,7 +965,7 @@ int lbm_step(lbm_sim *s, int64_t nsteps) {
   cudaStream_t st = s->mem.stream;
   for (int64_t k = 0; k < nsteps; ++k) {
     const StepArgs a = make_args(s);
-    cudaError_t e = launch_step(a, s->storage, s->layout, s->ns, (int)(s->t & 1), st);
+    cudaError_t e = launch_step(a, s->storage, s->layout, s->ns, (int)(s->t & 1), st, nullptr, k == 0, k == nsteps - 1);
     if (e != cudaSuccess) return cuda_fail(e, "step launch");
     s->t += 1;
   }
@@ -980,7 +981,7 @@ int lbm_step_timed(lbm_sim *s, float *ms, int64_t *entries) {
   for (int k = 0; k < 5 && e == cudaSuccess; ++k) e = cudaEventCreate(&ev[k]);
   if (e == cudaSuccess) {
     const StepArgs a = make_args(s);
-    e = launch_step(a, s->storage, s->layout, s->ns, (int)(s->t & 1), st, ev);
+    e = launch_step(a, s->storage, s->layout, s->ns, (int)(s->t & 1), st, ev, true, true);
     if (e == cudaSuccess) s->t += 1;
   }
   float em = 0.f, hm = 0.f;
@@ -1102,7 +1103,7 @@ int lbm_step_batch_mode(lbm_sim *const *sims, int n, int64_t nsteps, void *strea
       for (int q = 0; q < p.n_sims; ++q) p.t0[q] = sims[order[groups[gi].first + q]]->t + (done - p.k0);
       p.n_steps = (int32_t)m;
       const lbm_sim *s0 = sims[order[groups[gi].first]];
-      e = (m == 1 && !dsync) ? launch_batch_split(p, s0->storage, s0->layout, s0->ns, s0->det, st)
+      e = (m == 1 && !dsync) ? launch_batch_split(p, s0->storage, s0->layout, s0->ns, s0->det, st, done == 0, done == nsteps - 1)
                              : launch_batch(p, s0->storage, s0->layout, s0->ns, s0->det, st);
     }
     if (e == cudaSuccess && dsync && m > 1) {

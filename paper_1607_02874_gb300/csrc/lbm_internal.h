@@ -309,7 +309,7 @@ struct StepArgs {
   const int32_t *fcell;  // [n_lat] cell of each fluid entry (fluid-only layout)
   const float *inv_b;    // [n_nodes] 1 / b(node)
   const void *A_prev;    // [2][acc_row] species that reached the walls in the previous step (acc_t or float)
-  void *A_cur;           // [2][acc_row] written by this step's node_hits_kernel
+  void *A_cur;           // [2][acc_row] written by this step's hits (node_work)
   void *A_next;          // [2][acc_row] the ring's third buffer (unused by the step)
   const float *ub_prev;  // [2 sides][5][plane] u and species rho of planes 1 / nz-2, previous step
   float *ub_cur;         // same, written this step
@@ -524,13 +524,14 @@ struct BatchLaunch {
 static_assert(sizeof(BatchLaunch) <= 30720, "batched launch arguments too close to the kernel parameter limit");
 
 // Launch one step of parity (t & 1) for the given storage/layout/species:
-// the catalytic nodes' emission (node_emit_kernel), the fast kernel over
-// a.fast_list, the general kernel over a.gen_list, then the nodes' wall
-// hits (node_hits_kernel).
+// on the first step of a call the catalytic nodes' emission, the fast kernel
+// over a.fast_list, the general kernel over a.gen_list, then the nodes' wall
+// hits, with the next step's emission in the same launch unless this is the
+// last step of the call.
 // ev (optional, measurement): five events, recorded before the emission,
 // the fast kernel, the general kernel and the hits, and after the hits.
 cudaError_t launch_step(const StepArgs &a, int storage, int layout, int ns, int parity, cudaStream_t st,
-                        const cudaEvent_t *ev = nullptr);
+                        const cudaEvent_t *ev, bool first, bool last);
 // Per lattice warp: 0 no live entry, 1 plain, 2 general, 3 wall.
 cudaError_t launch_warp_class(const StepArgs &a, int layout, uint8_t *cls, int32_t *shift, cudaStream_t st);
 // RS: the random sputtering matrix; PHYS: the physics variant (kPhys*). Both
@@ -539,7 +540,8 @@ cudaError_t launch_warp_class(const StepArgs &a, int layout, uint8_t *cls, int32
 // in a translation unit of its own (step_*_rs.cu, step_*_bary.cu,
 // step_*_rs_bary.cu, step_*_chan.cu, step_*_rs_chan.cu).
 template <int ST, bool RS, int PHYS>
-cudaError_t launch_step_st(const StepArgs &a, int layout, int ns, int parity, cudaStream_t st, const cudaEvent_t *ev);
+cudaError_t launch_step_st(const StepArgs &a, int layout, int ns, int parity, cudaStream_t st, const cudaEvent_t *ev,
+                           bool first, bool last);
 __device__ __forceinline__ unsigned ld_acquire_gpu(const unsigned *p) {
   unsigned v;
   asm volatile("ld.acquire.gpu.global.u32 %0, [%1];" : "=r"(v) : "l"(p) : "memory");
@@ -591,11 +593,13 @@ struct BatchSync {
 // previous one. With p.n_steps > 1, p.sync must point to a zeroed BatchSync.
 template <int ST, bool RS, int PHYS>
 cudaError_t launch_batch_st(const BatchLaunch &p, int layout, int ns, int det, cudaStream_t st);
-// One step of every simulation in p (p.n_steps = 1) as four launches: the
-// emission of all catalytic nodes, the fast warps of all, the general warps
-// of all, then the wall hits of all nodes.
+// One step of every simulation in p (p.n_steps = 1): on the first step of a
+// call the emission of all catalytic nodes, the fast warps of all, the
+// general warps of all, then the wall hits of all nodes (with the next step's
+// emission unless this is the last step).
 template <int ST, bool RS, int PHYS>
-cudaError_t launch_batch_split_st(const BatchLaunch &p, int layout, int ns, int det, cudaStream_t st);
+cudaError_t launch_batch_split_st(const BatchLaunch &p, int layout, int ns, int det, cudaStream_t st, bool first,
+                                  bool last);
 
 // Observables: per-plane FP64 sums [nz][kPlaneCols] = rhoC, rhoR, rhoP,
 // rhoP*uz, hits R, hits P (last step).

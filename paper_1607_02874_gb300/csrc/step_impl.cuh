@@ -111,22 +111,28 @@ __device__ __forceinline__ int64_t hit_index(const StepArgs &a, int sp, int32_t 
          rs_rank(a.rs_key, node_cell, j, t, __ldg(a.node_off + LBM_OFF(a, kChkNode, 0, node + 1, a.n_nodes + 1)) - o);
 }
 
-// Species (R, P) re-emitted by the catalytic node `node` along its outgoing
-// link i (the incoming population of direction i of the fluid cell behind
-// it), in the units of the stored species (scaled deviations d = f / w).
-template <int ST, int NS, bool DET>
-__device__ __forceinline__ float2 emission(bool rs, const StepArgs &a, int i, int32_t node, int32_t node_cell) {
-  const float ib = __fmul_rn(emit_scale(rs, a, node), inv_wq(i) * Pop<ST, NS>::kSp);
-  const int64_t e = emit_index(rs, a, i, node, node_cell);
-  const float AR = acc_get<DET>(a.A_prev, LBM_OFF(a, kChkAcc, 0, e, LBM_NACC(a)));
+// What a node that gathered AR and AP re-emits along its outgoing link i, in
+// the units of the stored species (scaled deviations d = f / w); scale: the
+// link's share (1/b, or 1 under the random matrix, whose slots are per link).
+template <int ST, int NS>
+__device__ __forceinline__ float2 emission_of(const StepArgs &a, int i, float AR, float AP, float scale) {
+  const float ib = __fmul_rn(scale, inv_wq(i) * Pop<ST, NS>::kSp);
   float2 v;
   v.x = __fmul_rn(__fmul_rn(a.em_R, AR), ib);
   v.y = 0.0f;
-  if (NS > 2) {
-    const float AP = acc_get<DET>(a.A_prev, LBM_OFF(a, kChkAcc, 0, a.acc_row + e, LBM_NACC(a)));
-    v.y = __fmul_rn(fmaf(a.em_PR, AR, __fmul_rn(a.em_P, AP)), ib);
-  }
+  if (NS > 2) v.y = __fmul_rn(fmaf(a.em_PR, AR, __fmul_rn(a.em_P, AP)), ib);
   return v;
+}
+
+// Species (R, P) re-emitted by the catalytic node `node` along its outgoing
+// link i (the incoming population of direction i of the fluid cell behind
+// it), from the hits of the previous step.
+template <int ST, int NS, bool DET>
+__device__ __forceinline__ float2 emission(bool rs, const StepArgs &a, int i, int32_t node, int32_t node_cell) {
+  const int64_t e = emit_index(rs, a, i, node, node_cell);
+  const float AR = acc_get<DET>(a.A_prev, LBM_OFF(a, kChkAcc, 0, e, LBM_NACC(a)));
+  const float AP = NS > 2 ? acc_get<DET>(a.A_prev, LBM_OFF(a, kChkAcc, 0, a.acc_row + e, LBM_NACC(a))) : 0.0f;
+  return emission_of<ST, NS>(a, i, AR, AP, emit_scale(rs, a, node));
 }
 
 // Populations of lattice entry L at the current time as deviations
@@ -533,15 +539,27 @@ __device__ __forceinline__ int32_t flux_slot(const StepArgs &a, int32_t W) {
 }
 
 // Adds the warp's face flows, summed in FP64 in a fixed order, to its slot.
-// Every lane of the warp must call it.
+// Every lane of the warp must call it. The six sums are formed together: each
+// exchange halves the values a lane still carries (3, 2, 1, 1, 1 FP64 adds
+// instead of 6 x 5, on a chip whose FP64 pipe is slow), and the six lanes that
+// end with a sum add theirs to the slot at once.
 __device__ __forceinline__ void bank_flux(const StepArgs &a, int32_t W, const float (&flux)[6]) {
   const int32_t slot = flux_slot(a, W);
   if (slot < 0) return;
+  const int lane = threadIdx.x & 31;
+  const bool b4 = lane & 16, b3 = lane & 8, b2 = lane & 4;
+  double v[3];
 #pragma unroll
-  for (int k = 0; k < 6; ++k) {
-    const double v = warp_sum_d((double)flux[k]);
-    if ((threadIdx.x & 31) == 0) a.flux_cum[6 * (int64_t)slot + k] += v;
-  }
+  for (int k = 0; k < 3; ++k)
+    v[k] = (double)(b4 ? flux[k + 3] : flux[k]) + __shfl_xor_sync(0xffffffffu, (double)(b4 ? flux[k] : flux[k + 3]), 16);
+  const double u0 = (b3 ? v[2] : v[0]) + __shfl_xor_sync(0xffffffffu, b3 ? v[0] : v[2], 8);
+  const double u1 = v[1] + __shfl_xor_sync(0xffffffffu, v[1], 8);  // (of use where bit 3 is clear)
+  double w = (b2 && !b3 ? u1 : u0) + __shfl_xor_sync(0xffffffffu, b2 || b3 ? u0 : u1, 4);
+  w += __shfl_xor_sync(0xffffffffu, w, 2);
+  w += __shfl_xor_sync(0xffffffffu, w, 1);
+  // lanes 0, 4, 8 hold sums 0, 1, 2 and lanes 16, 20, 24 sums 3, 4, 5
+  if ((lane & 3) == 0 && (lane & 12) != 12)
+    a.flux_cum[6 * (int64_t)slot + (b4 ? 3 : 0) + ((lane >> 2) & 3)] += w;
 }
 
 // ---- Catalytic nodes: the sputtering law (Appendix, Eq. f_P_in) ----
@@ -552,13 +570,17 @@ __device__ __forceinline__ void bank_flux(const StepArgs &a, int32_t W, const fl
 // it reads from that same slot the population that arrives from n along c_j.
 // So the species part of the boundary acts on those slots alone, one thread
 // per node, around the cell updates of a step:
-//   node_emit, before them: bank the previous step's hits of the node, and
+//   emission, before them: bank the previous step's hits of the node, and
 //     write into each link's slot what the sputtering law returns along the
-//     link (emission);
-//   node_hits, after them: the species that reached the node in this step,
+//     link;
+//   hits, after them: the species that reached the node in this step,
 //     w_j times each link's stored value, summed over the node's links in a
 //     fixed order (or in 64-bit fixed point), into the step's accumulator
 //     (under the random matrix, each into the slot of the link it leaves by).
+// Between two steps of one call both fall to the same thread with nothing in
+// between, so one launch takes the hits of step t and the emission of step
+// t + 1 (kNodeBoth); the first step of a call emits alone and the last one
+// takes its hits alone, so that what a call leaves behind is always the hits.
 // The carrier's slot keeps its bounce-back. Inert solid is never a node, and
 // under species bounce-back (sp_bb) neither kernel runs, so the species
 // bounce back too.
@@ -585,11 +607,28 @@ __device__ __forceinline__ void link_entries(const StepArgs &a, int32_t nc, uint
   }
 }
 
-// Emission of node n for step t, and the banking of its previous hits into
-// hv (R, P). (t is passed apart from a.t: a batched launch reuses argument
-// sets six steps apart.)
-template <int ST, int LAYOUT, int NS, bool DET, bool RS>
-__device__ __forceinline__ void node_emit(const StepArgs &a, int64_t n, int64_t t, float (&hv)[2]) {
+// Node n around step t: MODE kNodeEmit, the emission of step t from the
+// previous step's hits; kNodeHits, the hits of step t into a.A_cur; kNodeBoth,
+// the hits of step t and then the emission of step t + 1 from them. hv: the
+// hits emitted from (R, P), to be banked. (t is passed apart from a.t: a
+// batched launch reuses argument sets six steps apart.)
+//
+// Bound by latency and by the 32-byte sectors around each link's 4-8 byte
+// slot. All of a node's links are issued together (one at a time took three
+// times as long on the 512x512x1024 sample); in kNodeBoth the links' entries
+// are found once and the slots are written while their lines are still in L2.
+// Node kernels per step, two launches before and one now: 531 -> 391 us
+// (512x512x1024, FP16, 7.6 M nodes), 80 -> 52 us (191x173x300, BF16, 0.93 M).
+constexpr int kNodeEmit = 1, kNodeHits = 2, kNodeBoth = 3;
+// Blocks per SM of the node kernels. kNodeBoth holds 18 entries and 18 loaded
+// slots: left to itself it takes 80-96 registers (2-3 blocks) and is slower
+// than the two launches it replaces (405 us a step on the 191x173x300 case).
+// Measured there at 4, 5 and 6 blocks: 379, 376 and 378 us; on the 512x512x1024
+// sample 9,082, 9,058 and 9,065; FP32 on 256x256x512 2,048, 2,054 and 2,051
+// (at 5 its fixed-point form spills 140 bytes, at 4 none).
+constexpr int node_min_blocks(int st, int mode) { return mode != kNodeBoth ? 1 : (st == LBM_FP32 ? 4 : 5); }
+template <int ST, int LAYOUT, int NS, bool DET, bool RS, int MODE>
+__device__ __forceinline__ void node_work(const StepArgs &a, int64_t n, int64_t t, float (&hv)[2]) {
   using P = Pop<ST, NS>;
   using STy = typename P::S;
   hv[0] = hv[1] = 0.f;
@@ -597,132 +636,127 @@ __device__ __forceinline__ void node_emit(const StepArgs &a, int64_t n, int64_t 
   const uint32_t links = __ldg(a.cell_bits + LBM_OFF(a, kChkIdx, 0, nc, LBM_NCELLS(a)));
   int32_t Ls[kQ];
   link_entries<LAYOUT>(a, nc, links, Ls);
-  if (RS) {
-    for (int32_t k = __ldg(a.node_off + LBM_OFF(a, kChkNode, 0, n, a.n_nodes + 1));
-         k < __ldg(a.node_off + LBM_OFF(a, kChkNode, 0, n + 1, a.n_nodes + 1)); ++k) {
-      hv[0] += acc_get<DET>(a.A_prev, LBM_OFF(a, kChkAcc, 0, k, LBM_NACC(a)));
-      if (NS > 2) hv[1] += acc_get<DET>(a.A_prev, LBM_OFF(a, kChkAcc, 0, a.acc_row + k, LBM_NACC(a)));
-    }
-  } else {
-    hv[0] = acc_get<DET>(a.A_prev, LBM_OFF(a, kChkAcc, 0, n, LBM_NACC(a)));
-    if (NS > 2) hv[1] = acc_get<DET>(a.A_prev, LBM_OFF(a, kChkAcc, 0, a.acc_row + n, LBM_NACC(a)));
-  }
   STy *const S = static_cast<STy *>(a.fs);
-  const uint32_t sd = step_seed_of(t, a.seed_mix);
+  int32_t o = 0, m = 0;  // random matrix: the node's link slots
+  if (RS) {
+    o = __ldg(a.node_off + LBM_OFF(a, kChkNode, 0, n, a.n_nodes + 1));
+    m = __ldg(a.node_off + LBM_OFF(a, kChkNode, 0, n + 1, a.n_nodes + 1)) - o;
+  }
+  // the hits that the emission works from: a.A_prev, or this thread's own
+  const void *const A = (MODE & kNodeHits) ? a.A_cur : a.A_prev;
+  if (MODE & kNodeHits) {
+    STy raw[kQ];
+#pragma unroll
+    for (int j = 1; j < kQ; ++j)
+      raw[j] = Ls[j] >= 0 ? S[LBM_OFF(a, kChkPop, 0, ent_off(Ls[j]) + 32 * j, LBM_NPOP(a))] : STy{};
+    if (RS)
+      for (int32_t k = 0; k < m; ++k) {
+        acc_clear<DET>(a.A_cur, LBM_OFF(a, kChkAcc, 0, o + k, LBM_NACC(a)));
+        if (NS > 2) acc_clear<DET>(a.A_cur, LBM_OFF(a, kChkAcc, 0, a.acc_row + o + k, LBM_NACC(a)));
+      }
+    acc_t iR = 0ull, iP = 0ull;  // fixed-point sums (DET)
+    float fR = 0.f, fP = 0.f;    // FP32 sums, in link order
+#pragma unroll
+    for (int j = 1; j < kQ; ++j) {
+      if (Ls[j] < 0) continue;
+      const float2 s = P::s_val(raw[j]);
+      // (the population that arrived moves along c_opp(j); w_opp(j) = w_j)
+      const float vR = __fmul_rn(wq(j) * P::kSpInv, s.x), vP = __fmul_rn(wq(j) * P::kSpInv, s.y);
+      if (RS) {
+        const int64_t k = o + rs_rank(a.rs_key, nc, opp(j), t, m);
+        acc_put<DET>(a.A_cur, LBM_OFF(a, kChkAcc, 0, k, LBM_NACC(a)), vR);
+        if (NS > 2) acc_put<DET>(a.A_cur, LBM_OFF(a, kChkAcc, 0, a.acc_row + k, LBM_NACC(a)), vP);
+      } else if (DET) {
+        iR += acc_from(vR);
+        if (NS > 2) iP += acc_from(vP);
+      } else {
+        fR = __fadd_rn(fR, vR);
+        if (NS > 2) fP = __fadd_rn(fP, vP);
+      }
+    }
+    if (!RS) {
+      if (DET) {
+        static_cast<acc_t *>(a.A_cur)[LBM_OFF(a, kChkAcc, 0, n, LBM_NACC(a))] = iR;
+        if (NS > 2) static_cast<acc_t *>(a.A_cur)[LBM_OFF(a, kChkAcc, 0, a.acc_row + n, LBM_NACC(a))] = iP;
+        hv[0] = acc_to_f(iR);
+        hv[1] = acc_to_f(iP);
+      } else {
+        static_cast<float *>(a.A_cur)[LBM_OFF(a, kChkAcc, 0, n, LBM_NACC(a))] = fR;
+        if (NS > 2) static_cast<float *>(a.A_cur)[LBM_OFF(a, kChkAcc, 0, a.acc_row + n, LBM_NACC(a))] = fP;
+        hv[0] = fR;
+        hv[1] = fP;
+      }
+    }
+  }
+  if (!(MODE & kNodeEmit)) return;
+  if (RS) {
+    for (int32_t k = o; k < o + m; ++k) {
+      hv[0] += acc_get<DET>(A, LBM_OFF(a, kChkAcc, 0, k, LBM_NACC(a)));
+      if (NS > 2) hv[1] += acc_get<DET>(A, LBM_OFF(a, kChkAcc, 0, a.acc_row + k, LBM_NACC(a)));
+    }
+  } else if (MODE == kNodeEmit) {
+    hv[0] = acc_get<DET>(A, LBM_OFF(a, kChkAcc, 0, n, LBM_NACC(a)));
+    if (NS > 2) hv[1] = acc_get<DET>(A, LBM_OFF(a, kChkAcc, 0, a.acc_row + n, LBM_NACC(a)));
+  }
+  const uint32_t sd = step_seed_of(MODE == kNodeBoth ? t + 1 : t, a.seed_mix);
+  const float scale = emit_scale(RS, a, (int32_t)n);
 #pragma unroll
   for (int j = 1; j < kQ; ++j) {
     if (Ls[j] < 0) continue;
-    const float2 v = emission<ST, NS, DET>(RS, a, j, (int32_t)n, nc);
+    float AR = hv[0], AP = hv[1];
+    if (RS) {  // (the link's rank among the node's active links)
+      const int64_t k = o + __popc(links & ((1u << j) - 1u));
+      AR = acc_get<DET>(A, LBM_OFF(a, kChkAcc, 0, k, LBM_NACC(a)));
+      if (NS > 2) AP = acc_get<DET>(A, LBM_OFF(a, kChkAcc, 0, a.acc_row + k, LBM_NACC(a)));
+    }
+    const float2 v = emission_of<ST, NS>(a, j, AR, AP, scale);
+    // (the slot's address is formed again from the entry, instead of the 18
+    // 64-bit addresses being held since the loads)
+    if (MODE == kNodeBoth) asm volatile("" : "+r"(Ls[j]));
     const uint32_t h = (ST == LBM_FP32) ? 0u : mix32(((uint32_t)Ls[j] + a.hash_base) ^ sd);
     S[LBM_OFF(a, kChkPop, 0, ent_off(Ls[j]) + 32 * j, LBM_NPOP(a))] = P::s_cv(v, h * sr_mul(2, j));
   }
 }
 
-// Wall hits of node n in step t: the species its links' cells sent towards
-// it, into a.A_cur.
-template <int ST, int LAYOUT, int NS, bool DET, bool RS>
-__device__ __forceinline__ void node_hits(const StepArgs &a, int64_t n, int64_t t) {
-  using P = Pop<ST, NS>;
-  using STy = typename P::S;
-  const int32_t nc = __ldg(a.node_cell + LBM_OFF(a, kChkNode, 0, n, a.n_nodes));
-  const uint32_t links = __ldg(a.cell_bits + LBM_OFF(a, kChkIdx, 0, nc, LBM_NCELLS(a)));
-  int32_t Ls[kQ];
-  link_entries<LAYOUT>(a, nc, links, Ls);
-  const STy *const S = static_cast<const STy *>(a.fs);
-  STy raw[kQ];
-#pragma unroll
-  for (int j = 1; j < kQ; ++j)
-    raw[j] = Ls[j] >= 0 ? S[LBM_OFF(a, kChkPop, 0, ent_off(Ls[j]) + 32 * j, LBM_NPOP(a))] : STy{};
-  int32_t o = 0, m = 0;
-  if (RS) {
-    o = __ldg(a.node_off + LBM_OFF(a, kChkNode, 0, n, a.n_nodes + 1));
-    m = __ldg(a.node_off + LBM_OFF(a, kChkNode, 0, n + 1, a.n_nodes + 1)) - o;
-    for (int32_t k = 0; k < m; ++k) {
-      acc_clear<DET>(a.A_cur, LBM_OFF(a, kChkAcc, 0, o + k, LBM_NACC(a)));
-      if (NS > 2) acc_clear<DET>(a.A_cur, LBM_OFF(a, kChkAcc, 0, a.acc_row + o + k, LBM_NACC(a)));
-    }
-  }
-  acc_t iR = 0ull, iP = 0ull;  // fixed-point sums (DET)
-  float fR = 0.f, fP = 0.f;    // FP32 sums, in link order
-#pragma unroll
-  for (int j = 1; j < kQ; ++j) {
-    if (Ls[j] < 0) continue;
-    const float2 s = P::s_val(raw[j]);
-    // (the population that arrived moves along c_opp(j); w_opp(j) = w_j)
-    const float vR = __fmul_rn(wq(j) * P::kSpInv, s.x), vP = __fmul_rn(wq(j) * P::kSpInv, s.y);
-    if (RS) {
-      const int64_t k = o + rs_rank(a.rs_key, nc, opp(j), t, m);
-      acc_put<DET>(a.A_cur, LBM_OFF(a, kChkAcc, 0, k, LBM_NACC(a)), vR);
-      if (NS > 2) acc_put<DET>(a.A_cur, LBM_OFF(a, kChkAcc, 0, a.acc_row + k, LBM_NACC(a)), vP);
-    } else if (DET) {
-      iR += acc_from(vR);
-      if (NS > 2) iP += acc_from(vP);
-    } else {
-      fR = __fadd_rn(fR, vR);
-      if (NS > 2) fP = __fadd_rn(fP, vP);
-    }
-  }
-  if (!RS) {
-    if (DET) {
-      static_cast<acc_t *>(a.A_cur)[LBM_OFF(a, kChkAcc, 0, n, LBM_NACC(a))] = iR;
-      if (NS > 2) static_cast<acc_t *>(a.A_cur)[LBM_OFF(a, kChkAcc, 0, a.acc_row + n, LBM_NACC(a))] = iP;
-    } else {
-      static_cast<float *>(a.A_cur)[LBM_OFF(a, kChkAcc, 0, n, LBM_NACC(a))] = fR;
-      if (NS > 2) static_cast<float *>(a.A_cur)[LBM_OFF(a, kChkAcc, 0, a.acc_row + n, LBM_NACC(a))] = fP;
-    }
-  }
-}
-
-// Block-wide FP64 sum of K per-thread values, fixed order; result valid in
-// thread 0. Must be called by every thread of the block.
-template <int K>
-__device__ __forceinline__ void block_sum_d(const float (&v)[K], double (&out)[K]) {
-  __shared__ double sh[K][kBlock / 32];
+// Adds the block's FP64 sums of a pair of per-thread values to dst[0] and
+// dst[1], in a fixed order: the first exchange leaves one value to each half
+// of the warp, then the 8 warps' pairs are summed by one warp. Must be called
+// by every thread of the block.
+__device__ __forceinline__ void bank_pair(const float (&v)[2], double *dst) {
+  __shared__ double sh[2][kBlock / 32];
   const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
+  const bool hi = lane & 16;
+  double s = (double)(hi ? v[1] : v[0]) + __shfl_xor_sync(0xffffffffu, (double)(hi ? v[0] : v[1]), 16);
 #pragma unroll
-  for (int k = 0; k < K; ++k) {
-    double s = warp_sum_d((double)v[k]);
-    if (lane == 0) sh[k][wid] = s;
-  }
+  for (int o = 8; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
+  if ((lane & 15) == 0) sh[lane >> 4][wid] = s;
   __syncthreads();
-  if (wid == 0) {
+  if (wid == 0 && lane < 2 * (kBlock / 32)) {
+    s = sh[lane / (kBlock / 32)][lane % (kBlock / 32)];
 #pragma unroll
-    for (int k = 0; k < K; ++k) {
-      double s = (lane < kBlock / 32) ? sh[k][lane] : 0.0;
-      s = warp_sum_d(s);
-      if (lane == 0) out[k] = s;
-    }
+    for (int o = kBlock / 64; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffu, s, o);
+    if (lane % (kBlock / 32) == 0) dst[lane / (kBlock / 32)] += s;
   }
-  __syncthreads();
 }
 
-// Node block blk (nodes blk 256 .. blk 256 + 255) of a node kernel: the
-// emission (banking the previous hits into the block's FP64 slot) or the
-// hits. Every thread of the block must call it.
-template <int ST, int LAYOUT, int NS, bool DET, bool RS, bool EMIT>
+// Node block blk (nodes blk 256 .. blk 256 + 255) of a node kernel; an
+// emission banks the hits it emits from into the block's FP64 slot. Every
+// thread of the block must call it.
+template <int ST, int LAYOUT, int NS, bool DET, bool RS, int MODE>
 __device__ __forceinline__ void node_block(const StepArgs &a, int blk, int64_t t) {
   if ((int64_t)blk * kBlock >= a.n_nodes) return;  // (uniform over the block)
   const int64_t n = (int64_t)blk * kBlock + threadIdx.x;
-  if (!EMIT) {
-    if (n < a.n_nodes) node_hits<ST, LAYOUT, NS, DET, RS>(a, n, t);
-    return;
-  }
   float hv[2] = {0.f, 0.f};
   if (n < a.n_nodes) {
-    node_emit<ST, LAYOUT, NS, DET, RS>(a, n, t, hv);
+    node_work<ST, LAYOUT, NS, DET, RS, MODE>(a, n, t, hv);
     if (n < a.bank_lo || n >= a.bank_hi) hv[0] = hv[1] = 0.f;  // (halo nodes are the neighbour's)
   }
-  double hs[2];
-  block_sum_d<2>(hv, hs);
-  if (threadIdx.x == 0) {
-    a.node_cum[2 * (int64_t)blk + 0] += hs[0];
-    a.node_cum[2 * (int64_t)blk + 1] += hs[1];
-  }
+  if (MODE & kNodeEmit) bank_pair(hv, a.node_cum + 2 * (int64_t)blk);
 }
 
-template <int ST, int LAYOUT, int NS, bool DET, bool RS, bool EMIT>
-__global__ void __launch_bounds__(kBlock) node_kernel(const StepArgs a) {
-  node_block<ST, LAYOUT, NS, DET, RS, EMIT>(a, (int)blockIdx.x, a.t);
+template <int ST, int LAYOUT, int NS, bool DET, bool RS, int MODE>
+__global__ void __launch_bounds__(kBlock, node_min_blocks(ST, MODE)) node_kernel(const StepArgs a) {
+  node_block<ST, LAYOUT, NS, DET, RS, MODE>(a, (int)blockIdx.x, a.t);
 }
 
 // Fast kernel: one warp per listed lattice warp. These warps need no
@@ -861,9 +895,9 @@ __global__ void __launch_bounds__(kBlock, kGenMinBlocks) batch_step_kernel(const
       step_block<ST, LAYOUT, NS, 0, DET, RS, PHYS>(a, blk, step);
   } else if (!a.sp_bb) {
     if (ph % 3 == 0)
-      node_block<ST, LAYOUT, NS, DET, RS, true>(a, blk, step);
+      node_block<ST, LAYOUT, NS, DET, RS, kNodeEmit>(a, blk, step);
     else
-      node_block<ST, LAYOUT, NS, DET, RS, false>(a, blk, step);
+      node_block<ST, LAYOUT, NS, DET, RS, kNodeHits>(a, blk, step);
   }
   __syncthreads();  // every thread's writes of this block precede the release
   if (threadIdx.x == 0) {
@@ -887,13 +921,13 @@ __device__ __forceinline__ int batch_owner(const int32_t *start, int n, int w) {
 
 // Per-step batched node kernels: node block w - node_start[q] of simulation
 // q, each at its own step.
-template <int ST, int LAYOUT, int NS, bool DET, bool RS, bool EMIT>
-__global__ void __launch_bounds__(kBlock) batch_node_kernel(const __grid_constant__ BatchLaunch p) {
+template <int ST, int LAYOUT, int NS, bool DET, bool RS, int MODE>
+__global__ void __launch_bounds__(kBlock, node_min_blocks(ST, MODE)) batch_node_kernel(const __grid_constant__ BatchLaunch p) {
   const int w = (int)blockIdx.x;
   const int q = batch_owner(p.node_start, p.n_sims, w);
   const StepArgs &a = p.v[q][p.k0 % 6];
   if (a.sp_bb) return;
-  node_block<ST, LAYOUT, NS, DET, RS, EMIT>(a, w - p.node_start[q], p.t0[q] + p.k0);
+  node_block<ST, LAYOUT, NS, DET, RS, MODE>(a, w - p.node_start[q], p.t0[q] + p.k0);
 }
 
 // Per-step batched launches, split as for a single simulation: the fast
@@ -1130,12 +1164,13 @@ __global__ void __launch_bounds__(kBlock) export_kernel(const StepArgs a, int wh
 // time) are compile-time parameters, so that the default kernels carry none
 // of the other modes' code.
 template <int ST, bool RS, int PHYS>
-cudaError_t launch_step_st(const StepArgs &a, int layout, int ns, int parity, cudaStream_t st, const cudaEvent_t *ev) {
+cudaError_t launch_step_st(const StepArgs &a, int layout, int ns, int parity, cudaStream_t st, const cudaEvent_t *ev,
+                           bool first, bool last) {
   if (ev) cudaEventRecord(ev[0], st);
   const unsigned ggrid = (unsigned)((a.n_gen + kWarpsPerBlock - 1) / kWarpsPerBlock);
   const unsigned ngrid = a.sp_bb ? 0u : (unsigned)((a.n_nodes + kBlock - 1) / kBlock);
-  if (ngrid > 0) {
-    LBM_DISPATCH_LNS(layout, ns, 0, a.det, node_kernel<ST, LY, NSC, DT, RS, true><<<ngrid, kBlock, 0, st>>>(a));
+  if (ngrid > 0 && first) {
+    LBM_DISPATCH_LNS(layout, ns, 0, a.det, node_kernel<ST, LY, NSC, DT, RS, kNodeEmit><<<ngrid, kBlock, 0, st>>>(a));
     const cudaError_t e = cudaGetLastError();
     if (e != cudaSuccess) return e;
   }
@@ -1170,8 +1205,12 @@ cudaError_t launch_step_st(const StepArgs &a, int layout, int ns, int parity, cu
     if (e != cudaSuccess) return e;
   }
   if (ev) cudaEventRecord(ev[3], st);
-  if (ngrid > 0)
-    LBM_DISPATCH_LNS(layout, ns, 0, a.det, node_kernel<ST, LY, NSC, DT, RS, false><<<ngrid, kBlock, 0, st>>>(a));
+  if (ngrid > 0) {
+    if (last)
+      LBM_DISPATCH_LNS(layout, ns, 0, a.det, node_kernel<ST, LY, NSC, DT, RS, kNodeHits><<<ngrid, kBlock, 0, st>>>(a));
+    else
+      LBM_DISPATCH_LNS(layout, ns, 0, a.det, node_kernel<ST, LY, NSC, DT, RS, kNodeBoth><<<ngrid, kBlock, 0, st>>>(a));
+  }
   if (ev) cudaEventRecord(ev[4], st);
   return cudaGetLastError();
 }
@@ -1187,11 +1226,12 @@ cudaError_t launch_batch_st(const BatchLaunch &p, int layout, int ns, int det, c
 }
 
 template <int ST, bool RS, int PHYS>
-cudaError_t launch_batch_split_st(const BatchLaunch &p, int layout, int ns, int det, cudaStream_t st) {
+cudaError_t launch_batch_split_st(const BatchLaunch &p, int layout, int ns, int det, cudaStream_t st, bool first,
+                                  bool last) {
   if (p.n_sims <= 0 || p.n_steps != 1) return cudaErrorInvalidValue;
-  if (p.total_node > 0) {
+  if (p.total_node > 0 && first) {
     LBM_DISPATCH_LNS(layout, ns, 0, det,
-                     batch_node_kernel<ST, LY, NSC, DT, RS, true><<<(unsigned)p.total_node, kBlock, 0, st>>>(p));
+                     batch_node_kernel<ST, LY, NSC, DT, RS, kNodeEmit><<<(unsigned)p.total_node, kBlock, 0, st>>>(p));
     const cudaError_t e = cudaGetLastError();
     if (e != cudaSuccess) return e;
   }
@@ -1209,9 +1249,14 @@ cudaError_t launch_batch_split_st(const BatchLaunch &p, int layout, int ns, int 
     const cudaError_t e = cudaGetLastError();
     if (e != cudaSuccess) return e;
   }
-  if (p.total_node > 0)
-    LBM_DISPATCH_LNS(layout, ns, 0, det,
-                     batch_node_kernel<ST, LY, NSC, DT, RS, false><<<(unsigned)p.total_node, kBlock, 0, st>>>(p));
+  if (p.total_node > 0) {
+    if (last)
+      LBM_DISPATCH_LNS(layout, ns, 0, det,
+                       batch_node_kernel<ST, LY, NSC, DT, RS, kNodeHits><<<(unsigned)p.total_node, kBlock, 0, st>>>(p));
+    else
+      LBM_DISPATCH_LNS(layout, ns, 0, det,
+                       batch_node_kernel<ST, LY, NSC, DT, RS, kNodeBoth><<<(unsigned)p.total_node, kBlock, 0, st>>>(p));
+  }
   return cudaGetLastError();
 }
 
@@ -1233,9 +1278,10 @@ cudaError_t launch_export_st(const StepArgs &a, int parity, int layout, int ns, 
 }
 
 #define LBM_INSTANTIATE_STEP(ST, RS, PHYS)                                                           \
-  template cudaError_t launch_step_st<ST, RS, PHYS>(const StepArgs &, int, int, int, cudaStream_t, const cudaEvent_t *); \
+  template cudaError_t launch_step_st<ST, RS, PHYS>(const StepArgs &, int, int, int, cudaStream_t, const cudaEvent_t *, \
+                                                          bool, bool);                                     \
   template cudaError_t launch_batch_st<ST, RS, PHYS>(const BatchLaunch &, int, int, int, cudaStream_t);   \
-  template cudaError_t launch_batch_split_st<ST, RS, PHYS>(const BatchLaunch &, int, int, int, cudaStream_t);
+  template cudaError_t launch_batch_split_st<ST, RS, PHYS>(const BatchLaunch &, int, int, int, cudaStream_t, bool, bool);
 #define LBM_INSTANTIATE_STORAGE(ST)                                                                    \
   LBM_INSTANTIATE_STEP(ST, false, kPhysCarrier)                                                               \
   template cudaError_t launch_plane_sums_st<ST>(const ObsArgs &, int, int, cudaStream_t);             \

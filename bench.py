@@ -3,11 +3,11 @@
 
 One "step" = one time step of the whole hot path (collision of carrier,
 reactant and product, streaming, bounce-back, catalytic sputtering,
-inlet/outlet planes, wall-hit bookkeeping) over every fluid cell: four
-launches (the catalytic nodes' emission, the fused collide-stream kernel
-over the warps away from the inlet/outlet planes, the one over the rest,
-the nodes' wall hits), five on odd steps, whose fast kernel takes the
-all-fluid region warps in a launch of their own. After the warm-up, --windows windows
+inlet/outlet planes, wall-hit bookkeeping) over every fluid cell: two
+launches (the fused collide-stream kernel over every cell; the catalytic
+nodes' wall hits with the next step's emission), three on odd steps, whose
+collide-stream kernel takes the all-fluid region warps in a launch of their
+own, and the first emission of a call. After the warm-up, --windows windows
 of --steps steps are timed; the line reports the median window.
 
 Prints one JSON line (rank 0). With --impl reference it times the FP64 CPU
@@ -468,15 +468,16 @@ def main():
                          f"{r['n_fluid']} fluid cells"}
 
     obs = res["obs"]
-    # launches in the timed windows: odd steps run the region warps' fast
-    # launch besides the one over the other fast warps
+    # launches in the timed windows, one call of --steps steps each: per step
+    # the cell kernel, a second one on odd steps for the region warps where
+    # there are 12,288 of them or more, and one node launch (the hits, with
+    # the next step's emission), besides the call's first emission
     wc = res["warps"]
-    other = int(e_gen > 0) + 2 * int(ginfo["n_nodes"] > 0)
     n_timed = args.steps * args.windows
     n_odd = (args.warmup + n_timed) // 2 - args.warmup // 2
-    fast_even = int(wc["plain"] + wc["region"] + wc["wall"] > 0)
-    fast_odd = int(wc["region"] > 0) + int(wc["plain"] + wc["wall"] > 0)
-    gpu_launches = (n_timed - n_odd) * (fast_even + other) + n_odd * (fast_odd + other)
+    region_launch = int(wc["region"] >= 12288)
+    node_launches = (n_timed + args.windows) * int(ginfo["n_nodes"] > 0)
+    gpu_launches = n_timed + n_odd * region_launch + node_launches
     line = {
         "metric": METRIC, "value": round(value, 1), "unit": "MLUPS", "n_gpus": world, "steps": args.steps,
         "warmup": args.warmup, "ms_per_step": round(ms_step, 4), "higher_is_better": True, "scaling": "weak",

@@ -62,6 +62,12 @@ constexpr int kUniShift = 26;
 constexpr uint32_t kWarpIdMask = (1u << kUniShift) - 1u;
 constexpr int kUniRegions = 31;
 constexpr int kUniTable = kUniRegions + 1;
+// Fewest region warps that take an odd launch of their own. Without the index
+// chain a region warp saves 0.16 ns (16-bit, 128x128x256) to 0.39 ns (FP32,
+// 256x256x512), and the launch costs 2.7 us (32x32x64: 12.3 us a step
+// without it, 13.6 with): the two meet at 7,000 to 17,000 warps. Below, the
+// region warps run with the others by the indexed addressing.
+constexpr int32_t kUniMinWarps = 12288;
 
 // D3Q19 speeds in the order documented in lbm.h. Written as constexpr
 // functions so that fully unrolled loops fold them into immediates.
@@ -524,12 +530,14 @@ struct BatchLaunch {
 static_assert(sizeof(BatchLaunch) <= 30720, "batched launch arguments too close to the kernel parameter limit");
 
 // Launch one step of parity (t & 1) for the given storage/layout/species:
-// on the first step of a call the catalytic nodes' emission, the fast kernel
-// over a.fast_list, the general kernel over a.gen_list, then the nodes' wall
-// hits, with the next step's emission in the same launch unless this is the
-// last step of the call.
-// ev (optional, measurement): five events, recorded before the emission,
-// the fast kernel, the general kernel and the hits, and after the hits.
+// on the first step of a call the catalytic nodes' emission, then the cell
+// kernel over the general warps (a.gen_list) and the fast ones (a.fast_list),
+// then the nodes' wall hits, with the next step's emission in the same launch
+// unless this is the last step of the call. The launches are chained
+// (chain_wait): one begins while the one before it drains.
+// ev (optional, measurement): five events, recorded before the emission, the
+// fast warps' launch, the general warps' (here two launches, one after the
+// other) and the hits, and after the hits.
 cudaError_t launch_step(const StepArgs &a, int storage, int layout, int ns, int parity, cudaStream_t st,
                         const cudaEvent_t *ev, bool first, bool last);
 // Per lattice warp: 0 no live entry, 1 plain, 2 general, 3 wall.

@@ -60,6 +60,16 @@ __device__ __forceinline__ int64_t ent_off(int32_t e) { return (int64_t)(e >> 5)
 // distance between two entries whenever that distance is below 2^31
 __device__ __forceinline__ uint32_t ent_off32(int32_t e) { return (uint32_t)e + ((uint32_t)e >> 5) * (uint32_t)(kQ * 32 - 32); }
 
+// The step's kernels follow one another on a stream with programmatic
+// dependent launch: each lets the next one be scheduled as soon as all its
+// own blocks have started (chain_next), and reads what earlier kernels wrote
+// only after they have completed (chain_wait). Before the wait a kernel may
+// read the lists and the geometry alone, which never change once a simulation
+// exists; so a launch's latency and the index loads overlap the kernel before
+// it. (Without the launch attribute both are no-ops.)
+__device__ __forceinline__ void chain_next() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
+__device__ __forceinline__ void chain_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
+
 // slots whose neighbour lies below / above the cell in z
 constexpr uint32_t kDownBits = (1u << 6) | (1u << 12) | (1u << 13) | (1u << 16) | (1u << 17);
 constexpr uint32_t kUpBits = (1u << 5) | (1u << 11) | (1u << 14) | (1u << 15) | (1u << 18);
@@ -210,8 +220,8 @@ __device__ __forceinline__ volatile int32_t &rel_slot(int k) {
 // whole warp lies away from the inlet/outlet and halo planes. Without WALL
 // it has no solid neighbour either; with WALL (nbm given) the odd step's
 // pointers of its solid links fall back to the cell's own reversed slot.
-template <int ST, int LAYOUT, int NS, int ODD, bool DET, bool FAST, bool RS, int PHYS, bool WALL = false,
-          bool SMEM = false, bool UNI = false>
+template <int ST, int LAYOUT, int NS, int ODD, bool FAST, int PHYS, bool WALL = false, bool SMEM = false,
+          bool UNI = false>
 __device__ __forceinline__ void cell_update(const StepArgs &a, int32_t L, int32_t cell, uint32_t nbm, int64_t t,
                                             float (&flux)[6]) {
   using P = Pop<ST, NS>;
@@ -281,6 +291,7 @@ __device__ __forceinline__ void cell_update(const StepArgs &a, int32_t L, int32_
       if constexpr (SREL) { if (k <= 16) rel_slot(k) = rel[k]; }
     }
   }
+  chain_wait();
   // ---- load ----
   // The 16-bit formats keep the species as loaded (one 32-bit register per
   // slot) and convert them where they are used, which holds 19 registers
@@ -642,6 +653,7 @@ __device__ __forceinline__ void node_work(const StepArgs &a, int64_t n, int64_t 
     o = __ldg(a.node_off + LBM_OFF(a, kChkNode, 0, n, a.n_nodes + 1));
     m = __ldg(a.node_off + LBM_OFF(a, kChkNode, 0, n + 1, a.n_nodes + 1)) - o;
   }
+  chain_wait();
   // the hits that the emission works from: a.A_prev, or this thread's own
   const void *const A = (MODE & kNodeHits) ? a.A_cur : a.A_prev;
   if (MODE & kNodeHits) {
@@ -756,18 +768,56 @@ __device__ __forceinline__ void node_block(const StepArgs &a, int blk, int64_t t
 
 template <int ST, int LAYOUT, int NS, bool DET, bool RS, int MODE>
 __global__ void __launch_bounds__(kBlock, node_min_blocks(ST, MODE)) node_kernel(const StepArgs a) {
+  chain_next();
   node_block<ST, LAYOUT, NS, DET, RS, MODE>(a, (int)blockIdx.x, a.t);
 }
 
-// Fast kernel: one warp per listed lattice warp. These warps need no
-// neighbour mask, no wall-hit accumulators and no face flows; even steps
-// touch only the entries' own slots. Even steps take the whole fast list in
-// one launch. Odd steps take it in two: the region warps at its head (UNI:
-// cell = entry + the region's shift, a word of the small table after the
-// lists, which stays in L1; no fcell, idx or nbm reads), then the rest.
+// General warp w of the list (solid neighbours, inlet/outlet planes, halo
+// planes).
+template <int ST, int LAYOUT, int NS, int ODD, int PHYS>
+__device__ __forceinline__ void gen_warp(const StepArgs &a, int w, int64_t t) {
+  const int32_t W = __ldg(a.gen_list + w);
+  const int32_t L = W * 32 + (threadIdx.x & 31);
+  float flux[6] = {0.f, 0.f, 0.f, 0.f, 0.f, 0.f};  // in C,R,P ; out C,R,P
+  if (L < a.n_lat) {
+    const int32_t cell = (LAYOUT == LBM_LAYOUT_DENSE) ? L : __ldg(a.fcell + L);
+    if ((LAYOUT != LBM_LAYOUT_DENSE || !__ldg(a.mask + cell)) && !halo_plane(a, cell / (a.nx * a.ny)))
+      cell_update<ST, LAYOUT, NS, ODD, false, PHYS>(a, L, cell, __ldg(a.nbm + L), t, flux);
+  }
+  bank_flux(a, W, flux);
+}
+
+// Cell kernel: one warp per listed lattice warp, the general warps in the
+// first blocks and the fast ones after them (block_0: the first block of that
+// sequence that this launch takes; list_0: the first fast warp). Fast warps
+// need no neighbour mask, no wall-hit accumulators and no face flows; even
+// steps touch only the entries' own slots. Even steps take the whole fast list
+// in one launch. Odd steps of large boxes take it in two: the region warps at
+// its head (UNI: cell = entry + the region's shift, a word of the small table
+// after the lists, which stays in L1; no fcell, idx or nbm reads), then the
+// rest.
+//
+// The general warps are 1-10 % of the warps and need 84-116 registers; in a
+// launch of their own they ran at 13 warps per SM after the fast warps had
+// drained. In the fast warps' launch they spill (96-230 bytes, in their branch
+// alone) but cost next to nothing. Step, with and without a launch of their
+// own: 158.5 and 161 us (128x128x256, FP16), 9,048 and 9,054 (512x512x1024,
+// FP16); 32x32x64 FP32 13.6 and 17.9 us.
 template <int ST, int LAYOUT, int NS, int ODD, int PHYS, bool UNI = false>
-__global__ void __launch_bounds__(kBlock, fast_min_blocks(ST, ODD)) fast_step_kernel(const StepArgs a) {
-  const int w = (ODD && !UNI ? a.n_uni : 0) + (int)blockIdx.x * kWarpsPerBlock + (int)(threadIdx.x >> 5);
+__global__ void __launch_bounds__(kBlock, fast_min_blocks(ST, ODD)) cell_kernel(const __grid_constant__ StepArgs a, int block_0,
+                                                                                        int list_0) {
+  chain_next();
+  int b = block_0 + (int)blockIdx.x;
+  if (!UNI) {
+    const int n_gen_blocks = (a.n_gen + kWarpsPerBlock - 1) / kWarpsPerBlock;
+    if (b < n_gen_blocks) {
+      const int w = b * kWarpsPerBlock + (int)(threadIdx.x >> 5);
+      if (w < a.n_gen) gen_warp<ST, LAYOUT, NS, ODD, PHYS>(a, w, a.t);
+      return;
+    }
+    b -= n_gen_blocks;
+  }
+  const int w = list_0 + b * kWarpsPerBlock + (int)(threadIdx.x >> 5);
   if (w >= (UNI ? a.n_uni : a.n_fast + a.n_wall)) return;
   const uint32_t v = (uint32_t)__ldg(a.fast_list + w);
   const int32_t L = (int32_t)(v & kWarpIdMask) * 32 + (threadIdx.x & 31);
@@ -784,33 +834,14 @@ __global__ void __launch_bounds__(kBlock, fast_min_blocks(ST, ODD)) fast_step_ke
   // odd steps: one code path for plain and wall warps, the solid-neighbour
   // mask being zero for a plain warp (two paths in one kernel spill more)
   const uint32_t nbm = (ODD && !UNI && (v & kWallWarp)) ? __ldg(a.nbm + L) : 0u;
-  cell_update<ST, LAYOUT, NS, ODD, false, true, false, PHYS, ODD != 0 && !UNI, true, UNI>(a, L, cell, nbm, a.t,
-                                                                                        flux);
-}
-
-// General kernel: one warp per listed lattice warp (solid neighbours,
-// inlet/outlet planes, halo planes).
-template <int ST, int LAYOUT, int NS, int ODD, bool DET, bool RS, int PHYS>
-__global__ void __launch_bounds__(kBlock, kGenMinBlocks) gen_step_kernel(const StepArgs a) {
-  const int w = blockIdx.x * kWarpsPerBlock + (threadIdx.x >> 5);
-  if (w < a.n_gen) {
-    const int32_t W = __ldg(a.gen_list + w);
-    const int32_t L = W * 32 + (threadIdx.x & 31);
-    float flux[6] = {0.f, 0.f, 0.f, 0.f, 0.f, 0.f};  // in C,R,P ; out C,R,P
-    if (L < a.n_lat) {
-      const int32_t cell = (LAYOUT == LBM_LAYOUT_DENSE) ? L : __ldg(a.fcell + L);
-      if ((LAYOUT != LBM_LAYOUT_DENSE || !__ldg(a.mask + cell)) && !halo_plane(a, cell / (a.nx * a.ny)))
-        cell_update<ST, LAYOUT, NS, ODD, DET, false, RS, PHYS>(a, L, cell, __ldg(a.nbm + L), a.t, flux);
-    }
-    bank_flux(a, W, flux);
-  }
+  cell_update<ST, LAYOUT, NS, ODD, true, PHYS, ODD != 0 && !UNI, true, UNI>(a, L, cell, nbm, a.t, flux);
 }
 
 // One step of the cells of one 256-entry block of lattice entries
 // (single-launch batches): each warp takes the fast path when all its live
 // entries can. Same arithmetic and face-flow slots as the fast and general
 // kernels.
-template <int ST, int LAYOUT, int NS, int ODD, bool DET, bool RS, int PHYS>
+template <int ST, int LAYOUT, int NS, int ODD, int PHYS>
 __device__ __forceinline__ void step_block(const StepArgs &a, const int blk, const int64_t t) {
   const int32_t L = (int32_t)(blk * kBlock + threadIdx.x);
   float flux[6] = {0.f, 0.f, 0.f, 0.f, 0.f, 0.f};  // in C,R,P ; out C,R,P
@@ -829,11 +860,11 @@ __device__ __forceinline__ void step_block(const StepArgs &a, const int blk, con
   const bool onplane = !live || (!halo && fast_plane(a, cell));
   live = live && !halo;
   if (__all_sync(0xffffffffu, plain) || (!ODD && __all_sync(0xffffffffu, onplane))) {
-    if (live) cell_update<ST, LAYOUT, NS, ODD, DET, true, RS, PHYS>(a, L, cell, 0u, t, flux);
+    if (live) cell_update<ST, LAYOUT, NS, ODD, true, PHYS>(a, L, cell, 0u, t, flux);
   } else if (__all_sync(0xffffffffu, onplane)) {  // a wall warp, odd step
-    if (live) cell_update<ST, LAYOUT, NS, ODD, DET, true, RS, PHYS, true>(a, L, cell, nbm, t, flux);
+    if (live) cell_update<ST, LAYOUT, NS, ODD, true, PHYS, true>(a, L, cell, nbm, t, flux);
   } else if (live) {
-    cell_update<ST, LAYOUT, NS, ODD, DET, false, RS, PHYS>(a, L, cell, nbm, t, flux);
+    cell_update<ST, LAYOUT, NS, ODD, false, PHYS>(a, L, cell, nbm, t, flux);
   }
   bank_flux(a, (int32_t)(L >> 5), flux);
 }
@@ -890,9 +921,9 @@ __global__ void __launch_bounds__(kBlock, kGenMinBlocks) batch_step_kernel(const
   const int blk = w - p.block_start[q];
   if (ph % 3 == 1) {
     if (a.parity)
-      step_block<ST, LAYOUT, NS, 1, DET, RS, PHYS>(a, blk, step);
+      step_block<ST, LAYOUT, NS, 1, PHYS>(a, blk, step);
     else
-      step_block<ST, LAYOUT, NS, 0, DET, RS, PHYS>(a, blk, step);
+      step_block<ST, LAYOUT, NS, 0, PHYS>(a, blk, step);
   } else if (!a.sp_bb) {
     if (ph % 3 == 0)
       node_block<ST, LAYOUT, NS, DET, RS, kNodeEmit>(a, blk, step);
@@ -957,7 +988,7 @@ __global__ void __launch_bounds__(kBlock, fast_min_blocks(ST, ODD)) batch_fast_k
   }
   float flux[6];
   const uint32_t nbm = (ODD && (v & kWallWarp)) ? __ldg(a.nbm + L) : 0u;
-  cell_update<ST, LAYOUT, NS, ODD, false, true, false, PHYS, ODD != 0, true>(a, L, cell, nbm, step, flux);
+  cell_update<ST, LAYOUT, NS, ODD, true, PHYS, ODD != 0, true>(a, L, cell, nbm, step, flux);
 }
 
 template <int ST, int LAYOUT, int NS, bool DET, bool RS, int PHYS>
@@ -976,9 +1007,9 @@ __global__ void __launch_bounds__(kBlock, kGenMinBlocks) batch_gen_kernel(const 
       const int32_t cell = (LAYOUT == LBM_LAYOUT_DENSE) ? L : __ldg(a.fcell + L);
       if ((LAYOUT != LBM_LAYOUT_DENSE || !__ldg(a.mask + cell)) && !halo_plane(a, cell / (a.nx * a.ny))) {
         if (a.parity)
-          cell_update<ST, LAYOUT, NS, 1, DET, false, RS, PHYS>(a, L, cell, __ldg(a.nbm + L), step, flux);
+          cell_update<ST, LAYOUT, NS, 1, false, PHYS>(a, L, cell, __ldg(a.nbm + L), step, flux);
         else
-          cell_update<ST, LAYOUT, NS, 0, DET, false, RS, PHYS>(a, L, cell, __ldg(a.nbm + L), step, flux);
+          cell_update<ST, LAYOUT, NS, 0, false, PHYS>(a, L, cell, __ldg(a.nbm + L), step, flux);
       }
     }
     bank_flux(a, W, flux);
@@ -1159,6 +1190,22 @@ __global__ void __launch_bounds__(kBlock) export_kernel(const StepArgs a, int wh
     else LBM_DISPATCH_N(LBM_LAYOUT_FLUID, NS_, ODD_, DET_, __VA_ARGS__);                   \
   } while (0)
 
+// A launch of the step's chain on st; overlap: it may begin before the kernel
+// ahead of it on the stream has completed (see chain_wait).
+template <typename... P, typename... A>
+cudaError_t launch_chained(void (*kernel)(P...), unsigned grid, cudaStream_t st, bool overlap, const A &...args) {
+  cudaLaunchAttribute at{};
+  at.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  at.val.programmaticStreamSerializationAllowed = 1;
+  cudaLaunchConfig_t c{};
+  c.gridDim = dim3(grid);
+  c.blockDim = dim3(kBlock);
+  c.stream = st;
+  c.attrs = &at;
+  c.numAttrs = overlap ? 1 : 0;
+  return cudaLaunchKernelEx(&c, kernel, args...);
+}
+
 // RS (the random sputtering matrix) and PHYS (carrier velocity; barycentric
 // velocity; validation channel: inert solid, body force, species relaxation
 // time) are compile-time parameters, so that the default kernels carry none
@@ -1169,50 +1216,53 @@ cudaError_t launch_step_st(const StepArgs &a, int layout, int ns, int parity, cu
   if (ev) cudaEventRecord(ev[0], st);
   const unsigned ggrid = (unsigned)((a.n_gen + kWarpsPerBlock - 1) / kWarpsPerBlock);
   const unsigned ngrid = a.sp_bb ? 0u : (unsigned)((a.n_nodes + kBlock - 1) / kBlock);
-  if (ngrid > 0 && first) {
-    LBM_DISPATCH_LNS(layout, ns, 0, a.det, node_kernel<ST, LY, NSC, DT, RS, kNodeEmit><<<ngrid, kBlock, 0, st>>>(a));
-    const cudaError_t e = cudaGetLastError();
-    if (e != cudaSuccess) return e;
-  }
+  const bool overlap = !ev;  // (timed apart, each launch waits for the one before)
+  cudaError_t e = cudaSuccess;
+  if (ngrid > 0 && first)
+    LBM_DISPATCH_LNS(layout, ns, 0, a.det, e = launch_chained(node_kernel<ST, LY, NSC, DT, RS, kNodeEmit>, ngrid, st, overlap, a));
+  if (e != cudaSuccess) return e;
   if (ev) cudaEventRecord(ev[1], st);
   // even steps: the whole fast list in one launch; odd steps: the region
-  // warps (fluid-only addressing), then the plain and wall warps in
-  // increasing order
-  const int32_t n_uni = (parity && layout == LBM_LAYOUT_FLUID) ? a.n_uni : 0;
+  // warps (fluid-only addressing, where there are enough of them), then the
+  // plain and wall warps in increasing order
+  const int32_t n_uni = (parity && layout == LBM_LAYOUT_FLUID && a.n_uni >= kUniMinWarps) ? a.n_uni : 0;
   if (n_uni > 0) {
     const unsigned ugrid = (unsigned)((n_uni + kWarpsPerBlock - 1) / kWarpsPerBlock);
     if (ns == 2)
-      fast_step_kernel<ST, LBM_LAYOUT_FLUID, 2, 1, PHYS, true><<<ugrid, kBlock, 0, st>>>(a);
+      e = launch_chained(cell_kernel<ST, LBM_LAYOUT_FLUID, 2, 1, PHYS, true>, ugrid, st, overlap, a, 0, 0);
     else
-      fast_step_kernel<ST, LBM_LAYOUT_FLUID, 3, 1, PHYS, true><<<ugrid, kBlock, 0, st>>>(a);
-    const cudaError_t e = cudaGetLastError();
+      e = launch_chained(cell_kernel<ST, LBM_LAYOUT_FLUID, 3, 1, PHYS, true>, ugrid, st, overlap, a, 0, 0);
     if (e != cudaSuccess) return e;
   }
   const unsigned fgrid =
       (unsigned)(((int64_t)a.n_fast + a.n_wall - n_uni + kWarpsPerBlock - 1) / kWarpsPerBlock);
-  if (fgrid > 0) {
+  auto cells = [&](unsigned block_0, unsigned blocks) {
+    if (blocks == 0) return cudaSuccess;
+    cudaError_t r;
     if (parity)
-      LBM_DISPATCH_LN(layout, ns, fast_step_kernel<ST, LY, NSC, 1, PHYS><<<fgrid, kBlock, 0, st>>>(a));
+      LBM_DISPATCH_LN(layout, ns, r = launch_chained(cell_kernel<ST, LY, NSC, 1, PHYS>, blocks, st, overlap, a, (int)block_0, n_uni));
     else
-      LBM_DISPATCH_LN(layout, ns, fast_step_kernel<ST, LY, NSC, 0, PHYS><<<fgrid, kBlock, 0, st>>>(a));
-    const cudaError_t e = cudaGetLastError();
+      LBM_DISPATCH_LN(layout, ns, r = launch_chained(cell_kernel<ST, LY, NSC, 0, PHYS>, blocks, st, overlap, a, (int)block_0, n_uni));
+    return r;
+  };
+  if (ev) {  // the fast and the general warps timed apart
+    e = cells(ggrid, fgrid);
     if (e != cudaSuccess) return e;
+    cudaEventRecord(ev[2], st);
+    e = cells(0, ggrid);
+  } else {
+    e = cells(0, ggrid + fgrid);
   }
-  if (ev) cudaEventRecord(ev[2], st);
-  if (ggrid > 0) {
-    LBM_DISPATCH_LNS(layout, ns, parity, a.det, gen_step_kernel<ST, LY, NSC, OD, DT, RS, PHYS><<<ggrid, kBlock, 0, st>>>(a));
-    const cudaError_t e = cudaGetLastError();
-    if (e != cudaSuccess) return e;
-  }
+  if (e != cudaSuccess) return e;
   if (ev) cudaEventRecord(ev[3], st);
   if (ngrid > 0) {
     if (last)
-      LBM_DISPATCH_LNS(layout, ns, 0, a.det, node_kernel<ST, LY, NSC, DT, RS, kNodeHits><<<ngrid, kBlock, 0, st>>>(a));
+      LBM_DISPATCH_LNS(layout, ns, 0, a.det, e = launch_chained(node_kernel<ST, LY, NSC, DT, RS, kNodeHits>, ngrid, st, overlap, a));
     else
-      LBM_DISPATCH_LNS(layout, ns, 0, a.det, node_kernel<ST, LY, NSC, DT, RS, kNodeBoth><<<ngrid, kBlock, 0, st>>>(a));
+      LBM_DISPATCH_LNS(layout, ns, 0, a.det, e = launch_chained(node_kernel<ST, LY, NSC, DT, RS, kNodeBoth>, ngrid, st, overlap, a));
   }
   if (ev) cudaEventRecord(ev[4], st);
-  return cudaGetLastError();
+  return e;
 }
 
 template <int ST, bool RS, int PHYS>

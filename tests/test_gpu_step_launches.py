@@ -72,3 +72,41 @@ def test_node_counts_around_a_block(n_nodes):
     for _ in range(7):
         b.step(1)
     _assert_same(a, b)
+
+
+def test_region_warps_with_and_without_their_own_launch():
+    """More region warps than the launch of their own needs (12,288) in one
+    box, none in the other: the open planes below the slab evolve alike."""
+    from paper_1607_02874_gb300 import lbm
+
+    nx, ny, nz = 128, 128, 64
+    out = []
+    for fluid in (lbm.LAYOUT_FLUID, lbm.LAYOUT_DENSE):  # dense addressing has no region warps
+        g = lbm.Geometry(nx, ny, nz, slab=(52, 60), porosity=0.6, corr_len=4.0, seed=5)
+        s = _sim(lbm, g, layout=fluid, p=0.3)
+        w = s.warp_counts()
+        assert (w["region"] >= 12288) == (fluid == lbm.LAYOUT_FLUID), w
+        s.step(9)
+        out.append((s.populations(), s.observables(site_map=True)["site_map"]))
+    for x, y in zip(*out):
+        np.testing.assert_array_equal(x, y)
+
+
+def test_steps_under_stream_capture():
+    """A captured call of two steps, replayed once, leaves what the call leaves."""
+    import torch
+    from paper_1607_02874_gb300 import lbm
+
+    st = torch.cuda.Stream()
+    g = lbm.Geometry(BOX["nx"], BOX["ny"], BOX["nz"], slab=BOX["slab"], porosity=BOX["porosity"],
+                     corr_len=BOX["corr_len"], seed=BOX["seed"], stream=st)
+    a, b = (_sim(lbm, g, layout=2, storage=1, stream=st) for _ in range(2))
+    graph = torch.cuda.CUDAGraph()
+    torch.cuda.synchronize()
+    with torch.cuda.graph(graph, stream=st):
+        a.step(2)
+    with torch.cuda.stream(st):
+        graph.replay()
+    b.step(2)
+    torch.cuda.synchronize()
+    _assert_same(a, b)

@@ -1134,7 +1134,7 @@ int lbm_observables(lbm_sim *s, lbm_obs *o) {
   int r = run_plane_sums(s, ps);
   if (r) return r;
   double red[8] = {0, 0, 0, 0, 0, 0, 0, 0};
-  LBM_CUDA_TRY(launch_sum_columns(s->node_cum, s->n_blocks, 2, s->red_out, st), "sum wall hits");
+  LBM_CUDA_TRY(launch_sum_columns(s->node_cum, node_blocks(g), 2, s->red_out, st), "sum wall hits");
   if (g->bc != LBM_BC_PERIODIC && s->n_flux_slots > 0)
     LBM_CUDA_TRY(launch_sum_columns(s->flux_cum, s->n_flux_slots, 6, s->red_out + 2, st), "sum face flows");
   else

@@ -673,6 +673,12 @@ struct lbm_geometry {
   int64_t *fl_plane_h = nullptr, *node_plane_h = nullptr;                            // host copies
 };
 
+namespace lbm {
+// Blocks of the node kernels: the slots of node_cum in use (the array has one
+// per lattice block at least; the others stay 0).
+inline int64_t node_blocks(const lbm_geometry *g) { return (g->n_nodes + kBlock - 1) / kBlock; }
+}  // namespace lbm
+
 struct lbm_sim {
   const lbm_geometry *g = nullptr;
   lbm_params prm{};

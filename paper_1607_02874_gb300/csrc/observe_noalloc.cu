@@ -51,42 +51,51 @@ static cudaError_t scratch_address(int dev, double **out) {
   return cudaSuccess;
 }
 
-// One thread: the same sums, in the same order, as lbm_observables does on
-// the host, so the two entry points agree to the last bit.
-__global__ void noalloc_finish_kernel(double *scr, int nz, int periodic, double react_coef) {
-  if (blockIdx.x != 0 || threadIdx.x != 0) return;
+// One block: the same sums, in the same order, as lbm_observables does on the
+// host, so the two entry points agree to the last bit. Each of the five sums
+// over the planes is one thread's chain of FP64 adds; the rows come to it
+// through shared memory, a tile at a time, and the other threads write the
+// profiles. (One thread alone, waiting for device memory at every plane, took
+// 90 us for boxes of 48-192 planes, half of the call.)
+constexpr int kFinishThreads = 192;
+__global__ void __launch_bounds__(kFinishThreads) noalloc_finish_kernel(double *scr, int nz, int periodic, double react_coef) {
+  constexpr int kTile = 256;
+  __shared__ double sh[kTile * kPlaneCols];
   const double *rows = scr;
   double *prof = scr + kNoAllocRows;
   const double *red = prof + kNoAllocProf;
   double *out = (double *)red + 8;
-  double M0 = 0, M1 = 0, M2 = 0, hR = red[0], hP = red[1];
-  double bad = 0.0;
-  for (int z = 0; z < nz; ++z) {
-    const double *row = rows + (size_t)kPlaneCols * z;
-    for (int k = 0; k < kPlaneCols; ++k)
-      if (row[k] != row[k]) bad = 1.0;
-    const bool bc = !periodic && (z == 0 || z == nz - 1);
-    if (bc) {
-      for (int k = 0; k < kNoAllocProfiles; ++k) prof[(size_t)k * LBM_NOALLOC_MAX_PLANES + z] = 0.0;
-      continue;
+  const int t = (int)threadIdx.x;
+  // thread k of the first five: M_C, M_R, M_P (columns 0-2), hits R, P
+  // (columns 4, 5, on top of the banked ones)
+  const int col = t < 3 ? t : t + 1;
+  double sum = (t == 3 || t == 4) ? red[t - 3] : 0.0;
+  bool bad = false;
+  for (int z0 = 0; z0 < nz; z0 += kTile) {
+    const int m = min(kTile, nz - z0);
+    __syncthreads();
+    for (int i = t; i < m * kPlaneCols; i += kFinishThreads) {
+      const double v = rows[(size_t)kPlaneCols * z0 + i];
+      sh[i] = v;
+      bad |= v != v;
+      const int z = z0 + i / kPlaneCols, k = i % kPlaneCols;
+      const double w = !periodic && (z == 0 || z == nz - 1) ? 0.0 : v;
+      if (k < 4) prof[(size_t)k * LBM_NOALLOC_MAX_PLANES + z] = w;
+      if (k == 4) prof[(size_t)4 * LBM_NOALLOC_MAX_PLANES + z] = w == 0.0 ? 0.0 : react_coef * w;
     }
-    M0 += row[0];
-    M1 += row[1];
-    M2 += row[2];
-    hR += row[4];
-    hP += row[5];
-    for (int k = 0; k < 4; ++k) prof[(size_t)k * LBM_NOALLOC_MAX_PLANES + z] = row[k];
-    prof[(size_t)4 * LBM_NOALLOC_MAX_PLANES + z] = react_coef * row[4];
+    __syncthreads();
+    if (t < 5)
+      for (int i = 0; i < m; ++i) {
+        const int z = z0 + i;
+        if (periodic || (z != 0 && z != nz - 1)) sum += sh[kPlaneCols * i + col];
+      }
   }
-  out[0] = M0;
-  out[1] = M1;
-  out[2] = M2;
-  out[3] = hR;
-  out[4] = hP;
-  out[5] = rows[(size_t)kPlaneCols * 1 + 1];         // sum rho_R, plane 1
-  out[6] = rows[(size_t)kPlaneCols * (nz - 2) + 2];  // sum rho_P, plane nz-2
-  out[7] = bad;
-  for (int k = 0; k < 6; ++k) out[8 + k] = red[2 + k];  // face flows
+  bad = __syncthreads_or(bad);
+  if (t < 5) out[t] = sum;
+  if (t == 5) out[5] = rows[(size_t)kPlaneCols * 1 + 1];         // sum rho_R, plane 1
+  if (t == 6) out[6] = rows[(size_t)kPlaneCols * (nz - 2) + 2];  // sum rho_P, plane nz-2
+  if (t == 7) out[7] = bad ? 1.0 : 0.0;
+  if (t < 6) out[8 + t] = red[2 + t];  // face flows
 }
 
 }  // namespace lbm
@@ -117,7 +126,7 @@ extern "C" int lbm_observables_noalloc(lbm_sim *s, lbm_obs *o) {
     e = launch_plane_sums(oa, s->storage, s->layout, s->ns, st);
   }
   double *red = scr + kNoAllocRows + kNoAllocProf;
-  if (e == cudaSuccess) e = launch_sum_columns(s->node_cum, s->n_blocks, 2, red, st);
+  if (e == cudaSuccess) e = launch_sum_columns(s->node_cum, node_blocks(g), 2, red, st);
   if (e == cudaSuccess) {
     if (g->bc != LBM_BC_PERIODIC && s->n_flux_slots > 0)
       e = launch_sum_columns(s->flux_cum, s->n_flux_slots, 6, red + 2, st);
@@ -126,7 +135,7 @@ extern "C" int lbm_observables_noalloc(lbm_sim *s, lbm_obs *o) {
   }
   const double coef = s->p * s->prm.pS_R;
   if (e == cudaSuccess) {
-    noalloc_finish_kernel<<<1, 1, 0, st>>>(scr, g->nz, g->bc == LBM_BC_PERIODIC, coef);
+    noalloc_finish_kernel<<<1, kFinishThreads, 0, st>>>(scr, g->nz, g->bc == LBM_BC_PERIODIC, coef);
     e = cudaGetLastError();
   }
   if (e == cudaSuccess) e = cudaMemcpyAsync(buf, red + 8, sizeof(double) * 14, cudaMemcpyDeviceToHost, st);

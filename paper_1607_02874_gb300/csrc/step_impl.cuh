@@ -45,6 +45,8 @@
 // move as one pair and relax with packed FP32x2 arithmetic.
 #pragma once
 
+#include <cooperative_groups.h>
+
 #include <algorithm>
 
 #include "lbm_internal.h"
@@ -145,25 +147,119 @@ __device__ __forceinline__ float2 emission(bool rs, const StepArgs &a, int i, in
   return emission_of<ST, NS>(a, i, AR, AP, emit_scale(rs, a, node));
 }
 
-// Populations of lattice entry L at the current time as deviations
-// g = f - w rho_ref (species unscaled), as a two-lattice scheme would hold
-// them (natural order), for a state of parity ODD (ODD = 1: the last
-// completed step was an even one). For the observables and exports.
+// Populations of lattice entry L at the current time, as a two-lattice scheme
+// would hold them (natural order), in the stored form (scaled deviations d,
+// species in the stored units; w d is the deviation g = f - w rho_ref), for a state of parity ODD (ODD = 1: the last
+// completed step was an even one). For the observables and exports. C, S: load
+// the carrier's, the species' (a reader of one of them moves 1/3 or 2/3 of
+// the bytes); what is not loaded is 0.
+//
+// Every address is formed without a branch and all loads are issued together;
+// a cell next to a catalytic solid then replaces the species that the wall
+// re-emits.
+template <int ST, int LAYOUT, int NS, int ODD, bool DET, bool C = true, bool S = true>
+__device__ __forceinline__ void load_cell(const StepArgs &a, int32_t L, int32_t cell, uint32_t nbm,
+                                          float (&d)[NS][kQ]) {
+  using P = Pop<ST, NS>;
+  const typename P::C *Cb = static_cast<const typename P::C *>(a.f);
+  const typename P::S *Sb = static_cast<const typename P::S *>(a.fs);
+  Nbr nb;
+  if (ODD || (S && NS > 1 && nbm)) {
+    const int z = (int)fast_div((uint32_t)cell, a.div_plane_m, a.div_sh & 0xffu, (a.div_sh >> 8) & 0xffu);
+    const int32_t xy = cell - z * a.nx * a.ny;
+    const int y = (int)fast_div((uint32_t)xy, a.div_nx_m, (a.div_sh >> 16) & 0xffu, a.div_sh >> 24);
+    nb = Nbr(cell, xy - y * a.nx, y, z, a.nx, a.ny, a.nz, a.periodic_z);
+  }
+  // the entry whose slot holds the population of direction i: odd states, the
+  // upwind one, unless it is solid; then, as on even states, the cell's own
+  // (with a solid upwind the cell's own reversed post-collision population
+  // sits in slot i in both parities)
+  int32_t from[kQ];
+#pragma unroll
+  for (int i = 0; i < kQ; ++i) {
+    from[i] = L;
+    if (ODD && i != 0) {
+      const int32_t src = nb.at(-cx(i), -cy(i), -cz(i));  // (a stepped cell's neighbours lie in the box)
+      const int32_t e = LAYOUT == LBM_LAYOUT_DENSE ? src : __ldg(a.idx + LBM_OFF(a, kChkIdx, 0, src, LBM_NCELLS(a)));
+      from[i] = ((nbm >> opp(i)) & 1u) ? L : e;
+    }
+  }
+  typename P::S sraw[kQ];
+#pragma unroll
+  for (int i = 0; i < kQ; ++i) {
+    const int slot = (ODD && i != 0 && !((nbm >> opp(i)) & 1u)) ? opp(i) : i;
+    const int64_t at = ent_off(from[i]) + 32 * slot;
+    d[0][i] = C ? P::c_val(ld_pop(Cb + LBM_OFF(a, kChkPop, 0, at, LBM_NPOP(a)))) : 0.0f;
+    if (NS > 1 && S) sraw[i] = ld_pop(Sb + LBM_OFF(a, kChkPop, 0, at, LBM_NPOP(a)));
+  }
+#pragma unroll
+  for (int i = 0; i < kQ; ++i) {
+    if (NS < 2) continue;
+    float2 s = make_float2(0.0f, 0.0f);
+    if (S) {
+      s = P::s_val(sraw[i]);
+      if (i != 0 && ((nbm >> opp(i)) & 1u)) {
+        const int32_t node_cell = nb.at(-cx(i), -cy(i), -cz(i));
+        const int32_t node = __ldg(a.idx + LBM_OFF(a, kChkIdx, 0, node_cell, LBM_NCELLS(a)));
+        // inert solid or species bounce-back: every array's own reversed
+        // population, as the carrier's
+        if (!(node < 0 || a.sp_bb)) s = emission<ST, NS, DET>(a.rs != 0, a, i, node, node_cell);
+      }
+    }
+    d[1][i] = s.x;
+    if (NS > 2) d[2][i] = s.y;
+  }
+}
+// Density deviation and momentum of array k (0 carrier, 1 R, 2 P) of such a
+// cell: each population w d rounded, then added.
+template <int ST, int NS>
+__device__ __forceinline__ float cell_density(const float (&d)[NS][kQ], int k) {
+  float r = 0.f;
+#pragma unroll
+  for (int i = 0; i < kQ; ++i) r = __fadd_rn(r, __fmul_rn(wq(i) * (k ? Pop<ST, NS>::kSpInv : 1.0f), d[k][i]));
+  return r;
+}
+// dir: 0 x, 1 y, 2 z
+template <int ST, int NS>
+__device__ __forceinline__ float cell_momentum(const float (&d)[NS][kQ], int k, int dir) {
+  float j = 0.f;
+#pragma unroll
+  for (int i = 0; i < kQ; ++i) {
+    // (directions with c = 0 stay in the sum: an infinity among them makes the
+    // velocity a NaN, by which the observables know a diverged state)
+    const int c = dir == 0 ? cx(i) : (dir == 1 ? cy(i) : cz(i));
+    j = __fadd_rn(j, __fmul_rn(c * wq(i) * (k ? Pop<ST, NS>::kSpInv : 1.0f), d[k][i]));
+  }
+  return j;
+}
+
+// The same, as deviations g (species unscaled), slot by slot, for the plane
+// sums. The compiler contracts some of these products with the sums that
+// follow, block of branches by block, and a plane's 10^5 cells round alike: an
+// order of its own here moves the FP64 sums by up to 1e-8 against those of
+// earlier runs. So the loads stay in this order; the branch-free form above
+// would take 1,485 us instead of 2,318 (FP16, odd, 256x256x512).
 template <int ST, int LAYOUT, int NS, int ODD, bool DET>
-__device__ __forceinline__ void load_cell(const StepArgs &a, int32_t L, const Nbr &nb, uint32_t nbm,
-                                          float (&f)[NS][kQ]) {
+__device__ __forceinline__ void load_cell_by_slot(const StepArgs &a, int32_t L, const Nbr &nb, uint32_t nbm,
+                                                  float (&f)[NS][kQ]) {
   using P = Pop<ST, NS>;
   const typename P::C *Cb = static_cast<const typename P::C *>(a.f);
   const typename P::S *Sb = static_cast<const typename P::S *>(a.fs);
   const int64_t own = ent_off(L);
+  // the entries of all upwind cells, looked up together ahead of the branches
+  int32_t up[kQ];
+#pragma unroll
+  for (int i = 1; i < kQ; ++i) {
+    up[i] = nb.at(-cx(i), -cy(i), -cz(i));
+    if (ODD && LAYOUT != LBM_LAYOUT_DENSE) up[i] = __ldg(a.idx + LBM_OFF(a, kChkIdx, 0, up[i], LBM_NCELLS(a)));
+  }
 #pragma unroll
   for (int i = 0; i < kQ; ++i) {
     const bool solid_up = (i != 0) && ((nbm >> opp(i)) & 1u);
     int64_t base = own;
     int slot = i;
     if (ODD && i != 0 && !solid_up) {
-      const int32_t src = nb.at(-cx(i), -cy(i), -cz(i));
-      base = ent_off(LAYOUT == LBM_LAYOUT_DENSE ? src : __ldg(a.idx + LBM_OFF(a, kChkIdx, 0, src, LBM_NCELLS(a))));
+      base = ent_off(up[i]);
       slot = opp(i);
     }
     // carrier: with a solid upwind, the cell's own reversed post-collision
@@ -1016,30 +1112,48 @@ __global__ void __launch_bounds__(kBlock, kGenMinBlocks) batch_gen_kernel(const 
   }
 }
 
-// Per-plane FP64 sums of the current state: one block per plane. Columns:
-// rho_C, rho_R, rho_P, rho_P u_z over the plane's fluid cells (u_z the
-// carrier's, or the barycentric one when a.bary), and the raw
-// wall hits A^R, A^P of the last step over the plane's catalytic nodes.
-// Inlet/outlet planes give zeros.
+// Per-plane FP64 sums of the current state: one cluster of kSumBlocks blocks
+// per plane, which share out its entries and nodes and add their partial sums
+// in rank order through distributed shared memory (no scratch in device
+// memory, the same order on every call). Columns: rho_C, rho_R, rho_P,
+// rho_P u_z over the plane's fluid cells (u_z the carrier's, or the
+// barycentric one when a.bary), and the raw wall hits A^R, A^P of the last
+// step over the plane's catalytic nodes. Inlet/outlet planes give zeros.
+//
+// Bound by the bytes of the populations, read once, and next to that by the
+// FP64 pipe (two lanes per SM): a cell costs four conversions, three adds and
+// one fused multiply-add; the ones of the densities are counted, not added.
+// One block per plane left few warps in flight and the chip to the last
+// blocks' tails: the whole call took 1,347 us on the 256x256x512 box (FP16,
+// even state), 5,249 (FP16, odd), 1,593 and 2,641 (FP32), now 917, 2,318, 1,248
+// and 1,683.
+constexpr int kSumBlocks = 8;  // (the largest portable cluster)
+// Blocks per SM. Odd states load slot by slot, so they want warps: FP16 3,100,
+// 2,318, 2,474 us at 3, 4, 5 blocks, FP32 1,772, 1,683, 2,377 (more blocks
+// spill). Even ones: FP16 1,026, 982, 917, 1,133 at 2, 3, 4, 5; FP32 1,248,
+// 1,261, 1,354 at 2, 3, 4.
+constexpr int sum_min_blocks(int st, int odd) { return !odd && st == LBM_FP32 ? 2 : 4; }
 template <int ST, int LAYOUT, int NS, int ODD, bool DET>
-__global__ void __launch_bounds__(kBlock) plane_sums_kernel(const ObsArgs o) {
+__global__ void __cluster_dims__(kSumBlocks, 1, 1) __launch_bounds__(kBlock, sum_min_blocks(ST, ODD)) plane_sums_kernel(const ObsArgs o) {
+  namespace cg = cooperative_groups;
+  const cg::cluster_group cluster = cg::this_cluster();
   const StepArgs &a = o.s;
-  const int z = blockIdx.x;
-  const int64_t plane = (int64_t)a.nx * a.ny;
+  const int z = (int)blockIdx.x / kSumBlocks, part = (int)blockIdx.x % kSumBlocks;
   const bool bc = (!a.periodic_z && (z == 0 || z == a.nz - 1)) || halo_plane(a, z);
   double s[kPlaneCols] = {0, 0, 0, 0, 0, 0};
   if (!bc) {
-    const int64_t lo = o.lat_plane[z], hi = o.lat_plane[z + 1];
-    for (int64_t Lw = lo + threadIdx.x; Lw < hi; Lw += kBlock) {
+    const int64_t hi = o.lat_plane[z + 1];
+    int cells = 0;
+    for (int64_t Lw = o.lat_plane[z] + part * kBlock + threadIdx.x; Lw < hi; Lw += kSumBlocks * kBlock) {
       const int32_t L = (int32_t)Lw;
-      const int32_t cell = (LAYOUT == LBM_LAYOUT_DENSE) ? L : a.fcell[L];
-      if (LAYOUT == LBM_LAYOUT_DENSE && a.mask[cell]) continue;
-      const int32_t xy = cell - z * (int32_t)plane;
-      const int y = xy / a.nx;
-      const int x = xy - y * a.nx;
-      const Nbr nb(cell, x, y, z, a.nx, a.ny, a.nz, a.periodic_z);
+      const int32_t cell = (LAYOUT == LBM_LAYOUT_DENSE) ? L : __ldg(a.fcell + L);
+      const uint32_t nbm = __ldg(a.nbm + L);
+      if (LAYOUT == LBM_LAYOUT_DENSE && __ldg(a.mask + cell)) continue;
+      const int32_t xy = cell - z * a.nx * a.ny;
+      const int y = (int)fast_div((uint32_t)xy, a.div_nx_m, (a.div_sh >> 16) & 0xffu, a.div_sh >> 24);
+      const Nbr nb(cell, xy - y * a.nx, y, z, a.nx, a.ny, a.nz, a.periodic_z);
       float f[NS][kQ];
-      load_cell<ST, LAYOUT, NS, ODD, DET>(a, L, nb, a.nbm[L], f);
+      load_cell_by_slot<ST, LAYOUT, NS, ODD, DET>(a, L, nb, nbm, f);
       float drho = 0.f, jz = 0.f, rR = 0.f, rP = 0.f, jzs = 0.f;
 #pragma unroll
       for (int i = 0; i < kQ; ++i) {
@@ -1050,21 +1164,25 @@ __global__ void __launch_bounds__(kBlock) plane_sums_kernel(const ObsArgs o) {
 #pragma unroll
         for (int sp = 1; sp < NS; ++sp) jzs += cz(i) * f[sp][i];
       }
-      s[0] += 1.0 + (double)drho;
-      s[1] += rR;
-      s[2] += rP;
+      ++cells;
+      s[0] += (double)drho;
+      s[1] += (double)rR;
       const float uz = a.bary ? (jz + jzs) / ((1.0f + drho) + (rR + rP)) : jz / (1.0f + drho) + 0.5f * a.g_z;
-      s[3] += (double)rP * (double)uz;
+      const double P = (double)rP;
+      s[2] += P;
+      s[3] = fma(P, (double)uz, s[3]);
     }
+    s[0] += (double)cells;
     if (NS > 1) {
-      for (int64_t k = o.node_plane[z] + threadIdx.x; k < o.node_plane[z + 1]; k += kBlock) {
+      for (int64_t k = o.node_plane[z] + part * kBlock + threadIdx.x; k < o.node_plane[z + 1]; k += kSumBlocks * kBlock) {
         s[4] += hits_d<DET>(a, 0, k);
         if (NS > 2) s[5] += hits_d<DET>(a, 1, k);
       }
     }
   }
-  // block reduction in FP64, fixed order
+  // FP64 sums in a fixed order: lanes, warps, then the cluster's blocks
   __shared__ double sh[kPlaneCols][kBlock / 32];
+  __shared__ double total[kPlaneCols];
   const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
 #pragma unroll
   for (int k = 0; k < kPlaneCols; ++k) {
@@ -1072,75 +1190,100 @@ __global__ void __launch_bounds__(kBlock) plane_sums_kernel(const ObsArgs o) {
     if (lane == 0) sh[k][wid] = v;
   }
   __syncthreads();
-  if (wid == 0) {
-#pragma unroll
-    for (int k = 0; k < kPlaneCols; ++k) {
-      double v = (lane < kBlock / 32) ? sh[k][lane] : 0.0;
-      v = warp_sum_d(v);
-      if (lane == 0) o.plane_sums[kPlaneCols * (int64_t)z + k] = v;
-    }
+  if (threadIdx.x < kPlaneCols) {
+    double v = 0.0;
+    for (int w = 0; w < kBlock / 32; ++w) v += sh[threadIdx.x][w];
+    total[threadIdx.x] = v;
   }
+  cluster.sync();
+  if (part == 0 && threadIdx.x < kPlaneCols) {
+    double v = 0.0;
+    for (int r = 0; r < kSumBlocks; ++r) v += *cluster.map_shared_rank(&total[threadIdx.x], r);
+    o.plane_sums[kPlaneCols * (int64_t)z + threadIdx.x] = v;
+  }
+  cluster.sync();  // (a block's shared memory lives until the sums are read)
+}
+
+// The species' momenta together, direction by direction.
+template <int ST, int NS>
+__device__ __forceinline__ float species_momentum(const float (&d)[NS][kQ], int dir) {
+  float j = 0.f;
+#pragma unroll
+  for (int i = 0; i < kQ; ++i)
+#pragma unroll
+    for (int k = 1; k < NS; ++k) {
+      const int c = dir == 0 ? cx(i) : (dir == 1 ? cy(i) : cz(i));
+      j = __fadd_rn(j, __fmul_rn(c * wq(i) * Pop<ST, NS>::kSpInv, d[k][i]));
+    }
+  return j;
+}
+
+// What an export reads: the carrier's populations, the species', or both
+// (all populations; the barycentric velocity).
+constexpr int kReadCarrier = 1, kReadSpecies = 2, kReadAll = 3;
+inline int export_reads(const StepArgs &a, int which) {
+  if (which < 0) return kReadAll;
+  if (which == LBM_FIELD_RHO_R || which == LBM_FIELD_RHO_P) return kReadSpecies;
+  const bool velocity = which == LBM_FIELD_UX || which == LBM_FIELD_UY || which == LBM_FIELD_UZ;
+  return velocity && a.bary ? kReadAll : kReadCarrier;
 }
 
 // Dense export of a field (which >= 0) or of all populations (which < 0).
-template <int ST, int LAYOUT, int NS, int ODD, bool DET>
-__global__ void __launch_bounds__(kBlock) export_kernel(const StepArgs a, int which, float *dst, int64_t n) {
+// Bound by the bytes of the arrays it reads, once the loads of a cell are in
+// flight together. 256x256x512, us per field, before (every reader took both
+// arrays, 80 registers) and now: carrier fields 1,094 -> 393 (FP32, even
+// state), 2,193 -> 527 (FP32, odd), 1,007 -> 306 and 3,094 -> 485 (FP16);
+// species 1,089 -> 714, 2,190 -> 888, 1,000 -> 472, 3,091 -> 689.
+// Blocks per SM, the fastest of those measured there (3-6): a carrier reader
+// at 5 or 6, a species reader at 4 or 5 unless its odd FP32 form spills (995
+// us at 4, 946 at 3), a reader of both at 3.
+constexpr int export_min_blocks(int st, int odd, int read) {
+  return read == kReadAll ? 3 : read == kReadCarrier ? (odd ? 6 : 5) : st == LBM_FP32 ? (odd ? 3 : 4) : (odd ? 4 : 5);
+}
+template <int ST, int LAYOUT, int NS, int ODD, bool DET, int READ>
+__global__ void __launch_bounds__(kBlock, export_min_blocks(ST, ODD, READ))
+    export_kernel(const StepArgs a, int which, float *dst, int64_t n) {
   const int64_t Lw = (int64_t)blockIdx.x * kBlock + threadIdx.x;
   if (Lw >= a.n_lat) return;
   const int32_t L = (int32_t)Lw;
-  const int32_t plane = a.nx * a.ny;
-  const int32_t cell = (LAYOUT == LBM_LAYOUT_DENSE) ? L : a.fcell[L];
-  if (LAYOUT == LBM_LAYOUT_DENSE && a.mask[cell]) return;
-  const int z = cell / plane;
+  const int32_t cell = (LAYOUT == LBM_LAYOUT_DENSE) ? L : __ldg(a.fcell + L);
+  const uint32_t nbm = __ldg(a.nbm + L);
+  if (LAYOUT == LBM_LAYOUT_DENSE && __ldg(a.mask + cell)) return;
+  const int z = (int)fast_div((uint32_t)cell, a.div_plane_m, a.div_sh & 0xffu, (a.div_sh >> 8) & 0xffu);
   // inlet/outlet planes hold no state of their own (their upwind cells lie
   // outside the box): leave them at 0
   if ((!a.periodic_z && (z == 0 || z == a.nz - 1)) || halo_plane(a, z)) return;
-  const int32_t xy = cell - z * plane;
-  const int y = xy / a.nx;
-  const int x = xy - y * a.nx;
-  const Nbr nb(cell, x, y, z, a.nx, a.ny, a.nz, a.periodic_z);
-  float f[NS][kQ];
-  load_cell<ST, LAYOUT, NS, ODD, DET>(a, L, nb, a.nbm[L], f);
-  if (which < 0) {
+  float d[NS][kQ];
+  load_cell<ST, LAYOUT, NS, ODD, DET, (READ & kReadCarrier) != 0, (READ & kReadSpecies) != 0>(a, L, cell, nbm, d);
+  if (READ == kReadAll && which < 0) {
 #pragma unroll
     for (int s = 0; s < NS; ++s)
 #pragma unroll
-      for (int i = 0; i < kQ; ++i) dst[(int64_t)(s * kQ + i) * n + cell] = f[s][i];
+      for (int i = 0; i < kQ; ++i) dst[(int64_t)(s * kQ + i) * n + cell] = wq(i) * (s ? Pop<ST, NS>::kSpInv : 1.0f) * d[s][i];
     return;
   }
-  // velocity: the carrier's, or the barycentric one over every array
-  float drho = 0.f, jx = 0.f, jy = 0.f, jz = 0.f, rs[3] = {0.f, 0.f, 0.f}, js[3] = {0.f, 0.f, 0.f};
-#pragma unroll
-  for (int i = 0; i < kQ; ++i) {
-    drho += f[0][i];
-    jx += cx(i) * f[0][i];
-    jy += cy(i) * f[0][i];
-    jz += cz(i) * f[0][i];
-#pragma unroll
-    for (int s = 1; s < NS; ++s) {
-      rs[s] += f[s][i];
-      js[0] += cx(i) * f[s][i];
-      js[1] += cy(i) * f[s][i];
-      js[2] += cz(i) * f[s][i];
-    }
-  }
-  const float rho = 1.0f + drho;
-  const float rho_u = a.bary ? rho + (rs[1] + rs[2]) : rho;
-  if (a.bary) {
-    jx += js[0];
-    jy += js[1];
-    jz += js[2];
-  }
   float v = 0.f;
-  switch (which) {
-    case LBM_FIELD_RHO_C: v = rho; break;
-    case LBM_FIELD_DRHO_C: v = drho; break;
-    case LBM_FIELD_RHO_R: v = rs[1]; break;
-    case LBM_FIELD_RHO_P: v = rs[2]; break;
-    case LBM_FIELD_UX: v = jx / rho_u; break;
-    case LBM_FIELD_UY: v = jy / rho_u; break;
-    case LBM_FIELD_UZ: v = a.bary ? jz / rho_u : jz / rho_u + 0.5f * a.g_z; break;
-    default: break;
+  if (READ == kReadSpecies) {
+    v = cell_density<ST, NS>(d, which == LBM_FIELD_RHO_R ? 1 : NS - 1);
+  } else {
+    const float drho = cell_density<ST, NS>(d, 0), rho = 1.0f + drho;
+    if (which == LBM_FIELD_RHO_C) {
+      v = rho;
+    } else if (which == LBM_FIELD_DRHO_C) {
+      v = drho;
+    } else {
+      // velocity: the carrier's, or the barycentric one over every array
+      float j[3];
+#pragma unroll
+      for (int k = 0; k < 3; ++k) {
+        j[k] = cell_momentum<ST, NS>(d, 0, k);
+        if (READ == kReadAll) j[k] += species_momentum<ST, NS>(d, k);
+      }
+      float over = rho;
+      if (READ == kReadAll) over = rho + (cell_density<ST, NS>(d, 1) + (NS > 2 ? cell_density<ST, NS>(d, NS - 1) : 0.f));
+      v = (which == LBM_FIELD_UX ? j[0] : which == LBM_FIELD_UY ? j[1] : j[2]) / over;
+      if (READ != kReadAll && which == LBM_FIELD_UZ) v += 0.5f * a.g_z;
+    }
   }
   dst[cell] = v;
 }
@@ -1312,7 +1455,7 @@ cudaError_t launch_batch_split_st(const BatchLaunch &p, int layout, int ns, int 
 
 template <int ST>
 cudaError_t launch_plane_sums_st(const ObsArgs &o, int layout, int ns, cudaStream_t st) {
-  LBM_DISPATCH_LNS(layout, ns, o.parity, o.s.det, plane_sums_kernel<ST, LY, NSC, OD, DT><<<o.s.nz, kBlock, 0, st>>>(o));
+  LBM_DISPATCH_LNS(layout, ns, o.parity, o.s.det, plane_sums_kernel<ST, LY, NSC, OD, DT><<<o.s.nz * kSumBlocks, kBlock, 0, st>>>(o));
   return cudaGetLastError();
 }
 
@@ -1322,8 +1465,21 @@ cudaError_t launch_export_st(const StepArgs &a, int parity, int layout, int ns, 
   const unsigned grid = (unsigned)((a.n_lat + kBlock - 1) / kBlock);
   if (grid == 0) return cudaSuccess;
   const int64_t n = (int64_t)a.nx * a.ny * a.nz;
-  LBM_DISPATCH_LNS(layout, ns, parity, a.det,
-                   export_kernel<ST, LY, NSC, OD, DT><<<grid, kBlock, 0, st>>>(a, which, dst, n));
+  switch (export_reads(a, which)) {
+    case kReadCarrier:  // (no wall hits: one form for either accumulator)
+      if (parity)
+        LBM_DISPATCH_LN(layout, ns, export_kernel<ST, LY, NSC, 1, false, kReadCarrier><<<grid, kBlock, 0, st>>>(a, which, dst, n));
+      else
+        LBM_DISPATCH_LN(layout, ns, export_kernel<ST, LY, NSC, 0, false, kReadCarrier><<<grid, kBlock, 0, st>>>(a, which, dst, n));
+      break;
+    case kReadSpecies:
+      LBM_DISPATCH_LNS(layout, ns, parity, a.det,
+                       export_kernel<ST, LY, NSC, OD, DT, kReadSpecies><<<grid, kBlock, 0, st>>>(a, which, dst, n));
+      break;
+    default:
+      LBM_DISPATCH_LNS(layout, ns, parity, a.det,
+                       export_kernel<ST, LY, NSC, OD, DT, kReadAll><<<grid, kBlock, 0, st>>>(a, which, dst, n));
+  }
   return cudaGetLastError();
 }
 

@@ -515,55 +515,51 @@ int lbm_create_geometry(const lbm_geometry_desc *d, void *stream, const lbm_allo
     g->mem.a = *alloc;
     g->mem.has = true;
   }
-  std::vector<uint8_t> hmask((size_t)n);
-  if (d->mask) {
-    // copy and check in one parallel pass
-    int64_t bad = 0, inert = 0;
-    const uint8_t *src = d->mask;
-    uint8_t *hm = hmask.data();
+  const bool on_device = sample_on_device(d);
+  std::vector<uint8_t> hmask(on_device ? 0 : (size_t)n);
+  if (!on_device) {
+    if (d->mask) {
+      // copy and check in one parallel pass
+      int64_t bad = 0, inert = 0;
+      const uint8_t *src = d->mask;
+      uint8_t *hm = hmask.data();
 #pragma omp parallel for reduction(+ : bad, inert) schedule(static)
-    for (int64_t c = 0; c < n; ++c) {
-      const uint8_t v = src[c];
-      hm[c] = v;
-      bad += v > 2;
-      inert += v == 2;
+      for (int64_t c = 0; c < n; ++c) {
+        const uint8_t v = src[c];
+        hm[c] = v;
+        bad += v > 2;
+        inert += v == 2;
+      }
+      if (bad) {
+        delete g;
+        return arg_fail("mask values must be 0 (fluid), 1 (catalytic solid) or 2 (inert solid)");
+      }
+      g->n_inert = inert;
+    } else
+      grf_mask(d->nx, d->ny, d->nz, d->slab_z0, d->slab_z1, d->porosity, d->corr_len, d->seed, hmask.data());
+    if (g->bc == LBM_BC_PRESSURE) {
+      for (int z : {0, 1, d->nz - 2, d->nz - 1}) {
+        if ((g->halo_lo && z < 2) || (g->halo_hi && z >= d->nz - 2)) continue;  // halo planes may hold solid
+        for (int64_t k = 0; k < g->plane; ++k)
+          if (hmask[(size_t)(z * g->plane + k)]) {
+            delete g;
+            return arg_fail("solid cell in an inlet/outlet plane or next to one (planes 0, 1, nz-2, nz-1)");
+          }
+      }
     }
-    if (bad) {
-      delete g;
-      return arg_fail("mask values must be 0 (fluid), 1 (catalytic solid) or 2 (inert solid)");
-    }
-    g->n_inert = inert;
-  } else
-    grf_mask(d->nx, d->ny, d->nz, d->slab_z0, d->slab_z1, d->porosity, d->corr_len, d->seed, hmask.data());
-  if (g->bc == LBM_BC_PRESSURE) {
-    for (int z : {0, 1, d->nz - 2, d->nz - 1}) {
-      if ((g->halo_lo && z < 2) || (g->halo_hi && z >= d->nz - 2)) continue;  // halo planes may hold solid
-      for (int64_t k = 0; k < g->plane; ++k)
-        if (hmask[(size_t)(z * g->plane + k)]) {
-          delete g;
-          return arg_fail("solid cell in an inlet/outlet plane or next to one (planes 0, 1, nz-2, nz-1)");
-        }
-    }
-  }
-  g->delta = chord_length(g->nx, g->ny, g->nz, g->z0, g->z1, hmask.data());
-  // geometry identity for checkpoints: FNV-1a (64-bit) of every 1 MiB chunk of
-  // the mask, in parallel, then FNV-1a of the chunk hashes in order
-  constexpr uint64_t kFnvBasis = 0xcbf29ce484222325ULL, kFnvPrime = 0x100000001b3ULL;
-  constexpr int64_t kChunk = (int64_t)1 << 20;
-  const int64_t n_chunks = (n + kChunk - 1) / kChunk;
-  std::vector<uint64_t> chunk_hash((size_t)n_chunks);
-  const uint8_t *hm = hmask.data();
+    g->delta = chord_length(g->nx, g->ny, g->nz, g->z0, g->z1, hmask.data());
+    const int64_t n_chunks = (n + kHashChunk - 1) / kHashChunk;
+    std::vector<uint64_t> chunk_hash((size_t)n_chunks);
+    const uint8_t *hm = hmask.data();
 #pragma omp parallel for schedule(static)
-  for (int64_t k = 0; k < n_chunks; ++k) {
-    uint64_t h = kFnvBasis;
-    const int64_t end = std::min(n, (k + 1) * kChunk);
-    for (int64_t c = k * kChunk; c < end; ++c) h = (h ^ hm[c]) * kFnvPrime;
-    chunk_hash[(size_t)k] = h;
+    for (int64_t k = 0; k < n_chunks; ++k) {
+      uint64_t h = kFnvBasis;
+      const int64_t end = std::min(n, (k + 1) * kHashChunk);
+      for (int64_t c = k * kHashChunk; c < end; ++c) h = (h ^ hm[c]) * kFnvPrime;
+      chunk_hash[(size_t)k] = h;
+    }
+    g->mask_hash = hash_of_chunks(chunk_hash);
   }
-  uint64_t hsh = kFnvBasis;
-  for (uint64_t v : chunk_hash)
-    for (int byte = 0; byte < 8; ++byte) hsh = (hsh ^ ((v >> (8 * byte)) & 0xffu)) * kFnvPrime;
-  g->mask_hash = hsh;
   cudaStream_t st = (cudaStream_t)stream;
   g->mask = (uint8_t *)g->mem.alloc((size_t)n);
   g->idx = (int32_t *)g->mem.alloc(sizeof(int32_t) * n);
@@ -574,8 +570,13 @@ int lbm_create_geometry(const lbm_geometry_desc *d, void *stream, const lbm_allo
     set_error("geometry allocation failed");
     return LBM_ERR_OOM;
   }
-  cudaError_t e = cudaMemcpyAsync(g->mask, hmask.data(), (size_t)n, cudaMemcpyHostToDevice, st);
-  if (e == cudaSuccess) e = cudaStreamSynchronize(st);  // hmask is pageable and leaves scope
+  cudaError_t e;
+  if (on_device) {
+    e = generate_sample(g, d->porosity, d->corr_len, st);
+  } else {
+    e = cudaMemcpyAsync(g->mask, hmask.data(), (size_t)n, cudaMemcpyHostToDevice, st);
+    if (e == cudaSuccess) e = cudaStreamSynchronize(st);  // hmask is pageable and leaves scope
+  }
   if (e == cudaSuccess) e = build_structures(g, st);
   if (e != cudaSuccess) {
     lbm_geometry_free(g);

@@ -8,8 +8,11 @@
 
 #include <string>
 #include <type_traits>
+#include <vector>
 
 #include "../../include/lbm.h"
+
+struct lbm_geometry;
 
 namespace lbm {
 
@@ -638,6 +641,20 @@ cudaError_t launch_site_map(const void *A_prev_R, int det, int64_t n_nodes, cons
 void grf_mask(int nx, int ny, int nz, int z0, int z1, double porosity, double corr_len, uint64_t seed,
               uint8_t *mask);
 double chord_length(int nx, int ny, int nz, int z0, int z1, const uint8_t *mask);
+// Whether the device generates the sample that d describes: a synthetic one
+// whose slab leaves open ends free (else the mask has to be looked at before
+// anything is built), with room for the scratch in the geometry's own arrays
+// (from about 2,100 cells) and lines that fit shared memory (6,400 cells).
+bool sample_on_device(const lbm_geometry_desc *d);
+// The mask of g's synthetic sample, its chord length and its hash, on the
+// device; g's mask, idx, b and nbm_dense are allocated (the last three serve as
+// scratch). Synchronises st.
+cudaError_t generate_sample(lbm_geometry *g, double porosity, double corr_len, cudaStream_t st);
+// geometry identity for checkpoints: FNV-1a (64-bit) of every 1 MiB chunk of
+// the mask, then FNV-1a of the chunk hashes in order
+constexpr unsigned long long kFnvBasis = 0xcbf29ce484222325ULL, kFnvPrime = 0x100000001b3ULL;
+constexpr int64_t kHashChunk = (int64_t)1 << 20;
+uint64_t hash_of_chunks(const std::vector<uint64_t> &chunk_hash);
 
 void set_error(const std::string &msg);
 

@@ -384,7 +384,7 @@ def main():
     roof = {"bound": "hbm", "achieved": round(achieved, 1), "peak": peak, "unit": "GB/s",
             "frac": round(achieved / peak, 4), "traffic": traffic, "peak_kind": peak_kind,
             "bytes_per_cell_update": B_alg, "units_per_launch": e_fast,
-            "kernel": "fast_step_kernel (fused collide/stream of every warp away from the inlet/outlet planes, "
+            "kernel": "cell_kernel (fused collide/stream of every warp away from the inlet/outlet planes, "
                       f"with the bounce-back redirection for cells touching a solid; {e_fast} of {e_fast + e_gen} "
                       "lattice entries; on odd steps two launches, the all-fluid region warps and the rest, "
                       "timed together)",

@@ -1031,7 +1031,10 @@ int lbm_step_batch_mode(lbm_sim *const *sims, int n, int64_t nsteps, void *strea
     return ((((sims[k]->storage * 4 + sims[k]->layout) * 4 + sims[k]->ns) * 2 + sims[k]->det) * 2 + sims[k]->rs) * 4 +
            sims[k]->phys;
   };
-  std::stable_sort(order.begin(), order.end(), [&](int x, int y) { return key(x) < key(y); });
+  // (the simulations of a group in two runs, by the parity of their step)
+  std::stable_sort(order.begin(), order.end(), [&](int x, int y) {
+    return key(x) != key(y) ? key(x) < key(y) : (sims[x]->t & 1) < (sims[y]->t & 1);
+  });
   std::vector<std::pair<int, int>> groups;
   for (int q = 0; q < n;) {
     int r = q;
@@ -1070,27 +1073,23 @@ int lbm_step_batch_mode(lbm_sim *const *sims, int n, int64_t nsteps, void *strea
     BatchLaunch &p = P[gi];
     std::memset(&p, 0, sizeof(p));
     p.n_sims = groups[gi].second - groups[gi].first;
-    int32_t total = 0, tf = 0, tg = 0, tn = 0;
+    int32_t total = 0, tn = 0;
+    int64_t region_warps = 0;
     for (int q = 0; q < p.n_sims; ++q) {
       const lbm_sim *sq = sims[order[groups[gi].first + q]];
       p.block_start[q] = total;
       total += (int32_t)sq->n_blocks;
-      p.fast_start[q] = tf;
-      tf += (sq->n_fast + sq->n_wall + kWarpsPerBlock - 1) / kWarpsPerBlock;
-      p.gen_start[q] = tg;
-      tg += (sq->n_gen + kWarpsPerBlock - 1) / kWarpsPerBlock;
       p.node_start[q] = tn;
-      tn += (int32_t)((sq->g->n_nodes + kBlock - 1) / kBlock);
+      tn += (int32_t)node_blocks(sq->g);
+      region_warps += sq->n_uni;
+      if ((sq->t & 1) == (sims[order[groups[gi].first]]->t & 1)) p.n_lead = q + 1;
       for (int j = 0; j < 6; ++j) p.v[q][j] = make_args_at(sq, sq->t + j);
     }
     p.block_start[p.n_sims] = total;
     p.total_blocks = total;
-    p.fast_start[p.n_sims] = tf;
-    p.gen_start[p.n_sims] = tg;
     p.node_start[p.n_sims] = tn;
-    p.total_fast = tf;
-    p.total_gen = tg;
     p.total_node = tn;
+    p.uni = region_warps >= kUniMinWarps;
     p.sync = dsync ? dsync + gi : nullptr;
   }
   std::vector<int> flags(ng);
@@ -1103,6 +1102,13 @@ int lbm_step_batch_mode(lbm_sim *const *sims, int n, int64_t nsteps, void *strea
       p.k0 = (int32_t)(done % 6);  // only k0 mod 6 and t0 + k0 matter
       for (int q = 0; q < p.n_sims; ++q) p.t0[q] = sims[order[groups[gi].first + q]]->t + (done - p.k0);
       p.n_steps = (int32_t)m;
+      for (int q = 0; q < p.n_sims; ++q) {
+        const StepArgs &a = p.v[q][p.k0];
+        const int32_t regions = a.parity && p.uni ? a.n_uni : 0;
+        const auto blocks = [](int32_t warps) { return (warps + kWarpsPerBlock - 1) / kWarpsPerBlock; };
+        p.uni_start[q + 1] = p.uni_start[q] + blocks(regions);
+        p.cell_start[q + 1] = p.cell_start[q] + blocks(a.n_gen) + blocks(a.n_fast + a.n_wall - regions);
+      }
       const lbm_sim *s0 = sims[order[groups[gi].first]];
       e = (m == 1 && !dsync) ? launch_batch_split(p, s0->storage, s0->layout, s0->ns, s0->det, st, done == 0, done == nsteps - 1)
                              : launch_batch(p, s0->storage, s0->layout, s0->ns, s0->det, st);

@@ -517,13 +517,15 @@ struct BatchLaunch {
   int32_t k0;
   int32_t n_steps;
   struct BatchSync *sync;
-  // per-step launches: blocks of the fast kernel (the fast warps) and of the
-  // general kernel (the general warps and the catalytic nodes) of each
-  // simulation, [fast_start[k], fast_start[k + 1]) and likewise
-  int32_t fast_start[kMaxBatch + 1];
-  int32_t gen_start[kMaxBatch + 1];
-  int32_t node_start[kMaxBatch + 1];  // blocks of the two catalytic-node kernels (256 nodes each)
-  int32_t total_fast, total_gen, total_node;
+  // per-step launches: each simulation's blocks [start[k], start[k + 1]) of
+  // the cell kernel (general and fast warps) at its parity of this step, of
+  // the odd steps' region warps (uni: in a launch of their own) and of the
+  // node kernels. Simulations 0 .. n_lead - 1 are at one parity, the others at
+  // the other.
+  int32_t cell_start[kMaxBatch + 1];
+  int32_t uni_start[kMaxBatch + 1];
+  int32_t node_start[kMaxBatch + 1];
+  int32_t n_lead, uni, total_node;
 };
 // Kernel parameters may hold up to 32,764 bytes (CUDA 12.1 and later). Measured
 // on GB300 (CUDA 13.0): with argument blocks of 32,696 bytes every
@@ -605,9 +607,9 @@ struct BatchSync {
 template <int ST, bool RS, int PHYS>
 cudaError_t launch_batch_st(const BatchLaunch &p, int layout, int ns, int det, cudaStream_t st);
 // One step of every simulation in p (p.n_steps = 1): on the first step of a
-// call the emission of all catalytic nodes, the fast warps of all, the
-// general warps of all, then the wall hits of all nodes (with the next step's
-// emission unless this is the last step).
+// call the emission of all catalytic nodes, the warps of the simulations at
+// one parity and of those at the other, then the wall hits of all nodes (with
+// the next step's emission unless this is the last step).
 template <int ST, bool RS, int PHYS>
 cudaError_t launch_batch_split_st(const BatchLaunch &p, int layout, int ns, int det, cudaStream_t st, bool first,
                                   bool last);

@@ -18,38 +18,24 @@ namespace lbm {
 
 constexpr int kQ = 19;
 constexpr int kBlock = 256;
-// Resident blocks per SM (256 threads each) that the register budgets of
-// the step kernels aim at: the fast kernel (the warps away from the
-// inlet/outlet and halo planes), per storage and parity, and the general
-// kernel (every other warp) and the single-launch batched kernel.
-// Measured on the 256x256x512 and 512x512x1024 C+R+P boxes: 16-bit even
-// steps are 2% faster at 4 blocks (64 registers) than at 3. With the odd
-// step's offsets in shared memory, 16-bit odd steps are 4% faster at 4
-// blocks (64 registers, 16 bytes of spill) than at 3, and FP32 odd steps
-// fastest at 3 (80 registers, no spill; 4 blocks spill 84 bytes and are 1%
-// slower). The general kernel is slower at 3 than at 2 in both storages.
-#ifndef LBM_FAST_EVEN_MINB
-#define LBM_FAST_EVEN_MINB 4
-#endif
-#ifndef LBM_FAST_EVEN_MINB_F32
-#define LBM_FAST_EVEN_MINB_F32 3
-#endif
-#ifndef LBM_FAST_ODD_MINB
-#define LBM_FAST_ODD_MINB 4
-#endif
-#ifndef LBM_FAST_ODD_MINB_F32
-#define LBM_FAST_ODD_MINB_F32 3
-#endif
-#ifndef LBM_GEN_MINB
-#define LBM_GEN_MINB 2
-#endif
-constexpr int kGenMinBlocks = LBM_GEN_MINB;
-
-constexpr int fast_min_blocks(int st, int odd) {
-  return odd ? (st == LBM_FP32 ? LBM_FAST_ODD_MINB_F32 : LBM_FAST_ODD_MINB)
-             : (st == LBM_FP32 ? LBM_FAST_EVEN_MINB_F32 : LBM_FAST_EVEN_MINB);
-}
-constexpr int kWarpsPerBlock = kBlock / 32;
+// Threads of a block of the cell kernels (one warp per listed lattice warp, no
+// work across warps). A block's registers come free with its last warp: at 256
+// threads 28 of the 32 warps that the budget admits were in flight, and odd
+// steps wait for memory. us a step at 64, 128, 256, 512 threads: 512x512x1024
+// FP16 8,818, 8,831, 9,048, 9,712; 191x173x300 BF16 361, 358, 365, 388;
+// 256x256x512 FP16 1,266, 1,268, 1,304, 1,393, FP32 2,028, 2,030, 2,042,
+// 2,160; 128x128x256 FP16 155.3, 155.1, 159.6, 171.5; 32x32x64 FP32 10.8,
+// 10.1, 10.8, 12.4.
+constexpr int kCellBlock = 128;
+constexpr int kWarpsPerBlock = kCellBlock / 32;
+// Resident blocks of the cell kernels per SM that their register budgets aim
+// at: 8 in the 16-bit formats (64 registers), 6 in FP32 (80 registers; at 7 and
+// 8 odd steps spill and the 256x256x512 step is 0.1 and 1.5 % slower). 16-bit
+// at 7, 8, 10: 256x256x512 FP16 1,290, 1,267, 1,457 us, 191x173x300 BF16 358,
+// 358, 383.
+constexpr int cell_min_blocks(int st) { return st == LBM_FP32 ? 6 : 8; }
+// Those of the single-launch batched kernel (256 threads).
+constexpr int kGenMinBlocks = 2;
 // Entries of the fast kernel's warp list: the lattice warp number in the low
 // 26 bits (lattice entries are int32, so at most 2^26 warps), a region
 // number in bits 26-30 and the wall mark in bit 31. Region r > 0 marks a

@@ -302,9 +302,9 @@ __device__ __forceinline__ float2 fma2(float2 a, float2 b, float2 c) { return __
 // This thread's shared-memory slot for the odd step's offset along c_k
 // (k = 1 .. 16): the warp's [16][32] slice of a block-wide array (volatile,
 // so that the store reads it back instead of keeping a register copy).
-// 16 KB per block, 64 KB for four blocks; the last two offsets stay in
+// 8 KB per block, 64 KB for eight blocks; the last two offsets stay in
 // registers. Measured on the 512x512x1024 box, 16-bit odd steps are 1.8%
-// faster than with all 18 offsets in shared memory (73.7 KB for four
+// faster than with all 18 offsets in shared memory (73.7 KB for eight
 // blocks), which leaves the SM less L1.
 __device__ __forceinline__ volatile int32_t &rel_slot(int k) {
   __shared__ int32_t s_rel[kWarpsPerBlock * 16 * 32];
@@ -366,7 +366,7 @@ __device__ __forceinline__ void cell_update(const StepArgs &a, int32_t L, int32_
   // Odd fast steps park 16 of the 18 offsets in shared memory (this warp's
   // [16][32] slice) until the store, instead of holding them in registers
   // across the arithmetic: with them the kernel needs 80 registers and
-  // spills, without them it fits the 64 of four blocks per SM.
+  // spills, without them it fits 64.
   constexpr bool SREL = ODD && FAST && SMEM;
   int32_t rel[kQ];
   const uint32_t own32 = ent_off32(L);
@@ -923,8 +923,8 @@ __device__ __forceinline__ void fast_warp(const StepArgs &a, int w, int64_t t) {
 // own: 158.5 and 161 us (128x128x256, FP16), 9,048 and 9,054 (512x512x1024,
 // FP16); 32x32x64 FP32 13.6 and 17.9 us.
 template <int ST, int LAYOUT, int NS, int ODD, int PHYS, bool UNI = false>
-__global__ void __launch_bounds__(kBlock, fast_min_blocks(ST, ODD)) cell_kernel(const __grid_constant__ StepArgs a, int block_0,
-                                                                                        int list_0) {
+__global__ void __launch_bounds__(kCellBlock, cell_min_blocks(ST))
+    cell_kernel(const __grid_constant__ StepArgs a, int block_0, int list_0) {
   chain_next();
   int b = block_0 + (int)blockIdx.x;
   if (!UNI) {
@@ -1078,7 +1078,7 @@ __global__ void __launch_bounds__(kBlock, node_min_blocks(ST, MODE)) batch_node_
 // over every block and no region launch; now 94.6. The launches do not overlap
 // as a single simulation's do: on that batch it is worth 0.7 %.
 template <int ST, int LAYOUT, int NS, int PHYS, int ODD, bool UNI = false>
-__global__ void __launch_bounds__(kBlock, fast_min_blocks(ST, ODD))
+__global__ void __launch_bounds__(kCellBlock, cell_min_blocks(ST))
     batch_cell_kernel(const __grid_constant__ BatchLaunch p, int sim_0) {
   const int32_t *const start = UNI ? p.uni_start : p.cell_start;
   const int w = start[sim_0] + (int)blockIdx.x;
@@ -1323,13 +1323,13 @@ __global__ void __launch_bounds__(kBlock, export_min_blocks(ST, ODD, READ))
 // A launch of the step's chain on st; overlap: it may begin before the kernel
 // ahead of it on the stream has completed (see chain_wait).
 template <typename... P, typename... A>
-cudaError_t launch_chained(void (*kernel)(P...), unsigned grid, cudaStream_t st, bool overlap, const A &...args) {
+cudaError_t launch_chained(void (*kernel)(P...), unsigned grid, int threads, cudaStream_t st, bool overlap, const A &...args) {
   cudaLaunchAttribute at{};
   at.id = cudaLaunchAttributeProgrammaticStreamSerialization;
   at.val.programmaticStreamSerializationAllowed = 1;
   cudaLaunchConfig_t c{};
   c.gridDim = dim3(grid);
-  c.blockDim = dim3(kBlock);
+  c.blockDim = dim3((unsigned)threads);
   c.stream = st;
   c.attrs = &at;
   c.numAttrs = overlap ? 1 : 0;
@@ -1349,7 +1349,7 @@ cudaError_t launch_step_st(const StepArgs &a, int layout, int ns, int parity, cu
   const bool overlap = !ev;  // (timed apart, each launch waits for the one before)
   cudaError_t e = cudaSuccess;
   if (ngrid > 0 && first)
-    LBM_DISPATCH_LNS(layout, ns, 0, a.det, e = launch_chained(node_kernel<ST, LY, NSC, DT, RS, kNodeEmit>, ngrid, st, overlap, a));
+    LBM_DISPATCH_LNS(layout, ns, 0, a.det, e = launch_chained(node_kernel<ST, LY, NSC, DT, RS, kNodeEmit>, ngrid, kBlock, st, overlap, a));
   if (e != cudaSuccess) return e;
   if (ev) cudaEventRecord(ev[1], st);
   // even steps: the whole fast list in one launch; odd steps: the region
@@ -1359,9 +1359,9 @@ cudaError_t launch_step_st(const StepArgs &a, int layout, int ns, int parity, cu
   if (n_uni > 0) {
     const unsigned ugrid = (unsigned)((n_uni + kWarpsPerBlock - 1) / kWarpsPerBlock);
     if (ns == 2)
-      e = launch_chained(cell_kernel<ST, LBM_LAYOUT_FLUID, 2, 1, PHYS, true>, ugrid, st, overlap, a, 0, 0);
+      e = launch_chained(cell_kernel<ST, LBM_LAYOUT_FLUID, 2, 1, PHYS, true>, ugrid, kCellBlock, st, overlap, a, 0, 0);
     else
-      e = launch_chained(cell_kernel<ST, LBM_LAYOUT_FLUID, 3, 1, PHYS, true>, ugrid, st, overlap, a, 0, 0);
+      e = launch_chained(cell_kernel<ST, LBM_LAYOUT_FLUID, 3, 1, PHYS, true>, ugrid, kCellBlock, st, overlap, a, 0, 0);
     if (e != cudaSuccess) return e;
   }
   const unsigned fgrid =
@@ -1370,9 +1370,9 @@ cudaError_t launch_step_st(const StepArgs &a, int layout, int ns, int parity, cu
     if (blocks == 0) return cudaSuccess;
     cudaError_t r;
     if (parity)
-      LBM_DISPATCH_LN(layout, ns, r = launch_chained(cell_kernel<ST, LY, NSC, 1, PHYS>, blocks, st, overlap, a, (int)block_0, n_uni));
+      LBM_DISPATCH_LN(layout, ns, r = launch_chained(cell_kernel<ST, LY, NSC, 1, PHYS>, blocks, kCellBlock, st, overlap, a, (int)block_0, n_uni));
     else
-      LBM_DISPATCH_LN(layout, ns, r = launch_chained(cell_kernel<ST, LY, NSC, 0, PHYS>, blocks, st, overlap, a, (int)block_0, n_uni));
+      LBM_DISPATCH_LN(layout, ns, r = launch_chained(cell_kernel<ST, LY, NSC, 0, PHYS>, blocks, kCellBlock, st, overlap, a, (int)block_0, n_uni));
     return r;
   };
   if (ev) {  // the fast and the general warps timed apart
@@ -1387,9 +1387,9 @@ cudaError_t launch_step_st(const StepArgs &a, int layout, int ns, int parity, cu
   if (ev) cudaEventRecord(ev[3], st);
   if (ngrid > 0) {
     if (last)
-      LBM_DISPATCH_LNS(layout, ns, 0, a.det, e = launch_chained(node_kernel<ST, LY, NSC, DT, RS, kNodeHits>, ngrid, st, overlap, a));
+      LBM_DISPATCH_LNS(layout, ns, 0, a.det, e = launch_chained(node_kernel<ST, LY, NSC, DT, RS, kNodeHits>, ngrid, kBlock, st, overlap, a));
     else
-      LBM_DISPATCH_LNS(layout, ns, 0, a.det, e = launch_chained(node_kernel<ST, LY, NSC, DT, RS, kNodeBoth>, ngrid, st, overlap, a));
+      LBM_DISPATCH_LNS(layout, ns, 0, a.det, e = launch_chained(node_kernel<ST, LY, NSC, DT, RS, kNodeBoth>, ngrid, kBlock, st, overlap, a));
   }
   if (ev) cudaEventRecord(ev[4], st);
   return e;
@@ -1412,7 +1412,7 @@ cudaError_t launch_batch_split_st(const BatchLaunch &p, int layout, int ns, int 
   cudaError_t e = cudaSuccess;
   const unsigned ngrid = (unsigned)p.total_node;
   if (ngrid > 0 && first)
-    LBM_DISPATCH_LNS(layout, ns, 0, det, e = launch_chained(batch_node_kernel<ST, LY, NSC, DT, RS, kNodeEmit>, ngrid, st, false, p));
+    LBM_DISPATCH_LNS(layout, ns, 0, det, e = launch_chained(batch_node_kernel<ST, LY, NSC, DT, RS, kNodeEmit>, ngrid, kBlock, st, false, p));
   if (e != cudaSuccess) return e;
   // the run of simulations at the first one's parity, then the others
   const int run[3] = {0, p.n_lead, p.n_sims};
@@ -1423,24 +1423,24 @@ cudaError_t launch_batch_split_st(const BatchLaunch &p, int layout, int ns, int 
     const unsigned ugrid = odd ? (unsigned)(p.uni_start[q1] - p.uni_start[q0]) : 0u;
     if (ugrid > 0) {  // (p.uni: fluid-only addressing)
       if (ns == 2)
-        e = launch_chained(batch_cell_kernel<ST, LBM_LAYOUT_FLUID, 2, PHYS, 1, true>, ugrid, st, false, p, q0);
+        e = launch_chained(batch_cell_kernel<ST, LBM_LAYOUT_FLUID, 2, PHYS, 1, true>, ugrid, kCellBlock, st, false, p, q0);
       else
-        e = launch_chained(batch_cell_kernel<ST, LBM_LAYOUT_FLUID, 3, PHYS, 1, true>, ugrid, st, false, p, q0);
+        e = launch_chained(batch_cell_kernel<ST, LBM_LAYOUT_FLUID, 3, PHYS, 1, true>, ugrid, kCellBlock, st, false, p, q0);
       if (e != cudaSuccess) return e;
     }
     const unsigned grid = (unsigned)(p.cell_start[q1] - p.cell_start[q0]);
     if (grid == 0) continue;
     if (odd)
-      LBM_DISPATCH_LN(layout, ns, e = launch_chained(batch_cell_kernel<ST, LY, NSC, PHYS, 1>, grid, st, false, p, q0));
+      LBM_DISPATCH_LN(layout, ns, e = launch_chained(batch_cell_kernel<ST, LY, NSC, PHYS, 1>, grid, kCellBlock, st, false, p, q0));
     else
-      LBM_DISPATCH_LN(layout, ns, e = launch_chained(batch_cell_kernel<ST, LY, NSC, PHYS, 0>, grid, st, false, p, q0));
+      LBM_DISPATCH_LN(layout, ns, e = launch_chained(batch_cell_kernel<ST, LY, NSC, PHYS, 0>, grid, kCellBlock, st, false, p, q0));
     if (e != cudaSuccess) return e;
   }
   if (ngrid > 0) {
     if (last)
-      LBM_DISPATCH_LNS(layout, ns, 0, det, e = launch_chained(batch_node_kernel<ST, LY, NSC, DT, RS, kNodeHits>, ngrid, st, false, p));
+      LBM_DISPATCH_LNS(layout, ns, 0, det, e = launch_chained(batch_node_kernel<ST, LY, NSC, DT, RS, kNodeHits>, ngrid, kBlock, st, false, p));
     else
-      LBM_DISPATCH_LNS(layout, ns, 0, det, e = launch_chained(batch_node_kernel<ST, LY, NSC, DT, RS, kNodeBoth>, ngrid, st, false, p));
+      LBM_DISPATCH_LNS(layout, ns, 0, det, e = launch_chained(batch_node_kernel<ST, LY, NSC, DT, RS, kNodeBoth>, ngrid, kBlock, st, false, p));
   }
   return e;
 }

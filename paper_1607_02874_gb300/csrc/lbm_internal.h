@@ -121,6 +121,7 @@ struct Pop<LBM_FP32, NS> {
   using S = typename std::conditional<NS == 3, float2, float>::type;
   static constexpr float kSp = 1.0f, kSpInv = 1.0f;
   __device__ __forceinline__ static float c_val(C q) { return q; }
+  __device__ __forceinline__ static float c_half(uint32_t, bool) { return 0.0f; }
   __device__ __forceinline__ static float2 s_val(S q) {
     if constexpr (NS == 3) return q; else return make_float2(q, 0.0f);
   }
@@ -147,6 +148,8 @@ struct Pop<LBM_FP16_DEV, NS> {
   using S = typename std::conditional<NS == 3, unsigned, unsigned short>::type;
   static constexpr float kSp = 16384.0f, kSpInv = 1.0f / 16384.0f;  // 2^14, exact
   __device__ __forceinline__ static float c_val(C q) { return __half2float(__ushort_as_half(q)); }
+  // the lower or the upper one of a pair of carrier values in one register
+  __device__ __forceinline__ static float c_half(uint32_t r, bool hi) { return c_val((C)(hi ? r >> 16 : r & 0xffffu)); }
   __device__ __forceinline__ static float2 s_val(S q) {
     if constexpr (NS == 3) {
       __half2 h;
@@ -169,6 +172,7 @@ struct Pop<LBM_BF16_DEV, NS> {
   using S = typename std::conditional<NS == 3, unsigned, unsigned short>::type;
   static constexpr float kSp = 1.0f, kSpInv = 1.0f;
   __device__ __forceinline__ static float c_val(C q) { return __uint_as_float((uint32_t)q << 16); }
+  __device__ __forceinline__ static float c_half(uint32_t r, bool hi) { return __uint_as_float(hi ? r & 0xffff0000u : r << 16); }
   __device__ __forceinline__ static float2 s_val(S q) {
     if constexpr (NS == 3) return make_float2(__uint_as_float(q << 16), __uint_as_float(q & 0xffff0000u));
     else return make_float2(__uint_as_float((uint32_t)q << 16), 0.0f);

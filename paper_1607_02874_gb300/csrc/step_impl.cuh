@@ -300,15 +300,31 @@ __device__ __forceinline__ float2 add2(float2 a, float2 b) { return __fadd2_rn(a
 __device__ __forceinline__ float2 fma2(float2 a, float2 b, float2 c) { return __ffma2_rn(a, b, c); }
 
 // This thread's shared-memory slot for the odd step's offset along c_k
-// (k = 1 .. 16): the warp's [16][32] slice of a block-wide array (volatile,
-// so that the store reads it back instead of keeping a register copy).
-// 8 KB per block, 64 KB for eight blocks; the last two offsets stay in
-// registers. Measured on the 512x512x1024 box, 16-bit odd steps are 1.8%
-// faster than with all 18 offsets in shared memory (73.7 KB for eight
-// blocks), which leaves the SM less L1.
+// (k = 1 .. REL): the warp's [REL][32] slice of a block-wide array (volatile,
+// so that the store reads it back instead of keeping a register copy). The
+// offsets beyond REL stay in registers.
+//
+// With kRelNear of them a block takes 6 KB and eight fit the 64 KB that the
+// launch asks for, which leaves the SM 192 KB of L1 for the gathers; with 16
+// (8 KB, 100 KB asked for) the loads wait for more of the offsets, and odd
+// steps keep less in flight. us of the odd step's cells, kRelWide (in the 135
+// KB that the driver chose by itself) and kRelNear: 191x173x300 BF16 387 and
+// 332, 128x128x256 FP16 171 and 165, 256x256x512 FP16 1,377 and 1,352;
+// 10 and 14 are slower than 12 (341 and 344 on the first).
+//
+// Where the planes are large that turns round: the rows between the first and
+// the last warp in flight, with the planes above and below them, outgrow L2.
+// us a step of 16-bit boxes, three planes' populations in MB, kRelNear and
+// kRelWide: 26 MB (320x320) 1,432 and 1,454; 33 (512x256) 1,861 and 1,863; 37
+// (384x384) 2,089 and 2,085; 51 (448x448) 2,130 and 2,131; 66 (512x512) 2,759
+// and 2,747; 161 (800x800) 2,822 and 2,792; 66 (512x512x1024) 8,898 and 8,817.
+// FP32 keeps to kRelNear (512x512x300: 4,420 and 4,442), as do batches.
+constexpr int kRelNear = 12, kRelWide = 16;
+constexpr int64_t kWidePlanes = (int64_t)48 << 20;  // bytes, where the two meet
+template <int REL>
 __device__ __forceinline__ volatile int32_t &rel_slot(int k) {
-  __shared__ int32_t s_rel[kWarpsPerBlock * 16 * 32];
-  return *((volatile int32_t *)s_rel + (threadIdx.x >> 5) * (16 * 32) + (k - 1) * 32 + (threadIdx.x & 31));
+  __shared__ int32_t s_rel[kWarpsPerBlock * REL * 32];
+  return *((volatile int32_t *)s_rel + (threadIdx.x >> 5) * (REL * 32) + (k - 1) * 32 + (threadIdx.x & 31));
 }
 
 // Update of one cell: load the 19 slots of both arrays, moments, relaxation
@@ -316,7 +332,7 @@ __device__ __forceinline__ volatile int32_t &rel_slot(int k) {
 // whole warp lies away from the inlet/outlet and halo planes. Without WALL
 // it has no solid neighbour either; with WALL (nbm given) the odd step's
 // pointers of its solid links fall back to the cell's own reversed slot.
-template <int ST, int LAYOUT, int NS, int ODD, bool FAST, int PHYS, bool WALL = false, bool SMEM = false,
+template <int ST, int LAYOUT, int NS, int ODD, bool FAST, int PHYS, bool WALL = false, int REL = 0,
           bool UNI = false>
 __device__ __forceinline__ void cell_update(const StepArgs &a, int32_t L, int32_t cell, uint32_t nbm, int64_t t,
                                             float (&flux)[6]) {
@@ -363,11 +379,11 @@ __device__ __forceinline__ void cell_update(const StepArgs &a, int32_t L, int32_
   // outside neighbour, to the cell's own reversed slot. One 32-bit value per
   // slot; the node number of a solid neighbour is read again from idx where
   // a wall link needs it.
-  // Odd fast steps park 16 of the 18 offsets in shared memory (this warp's
-  // [16][32] slice) until the store, instead of holding them in registers
+  // Odd fast steps park REL of the 18 offsets in shared memory (this warp's
+  // [REL][32] slice) until the store, instead of holding them in registers
   // across the arithmetic: with them the kernel needs 80 registers and
   // spills, without them it fits 64.
-  constexpr bool SREL = ODD && FAST && SMEM;
+  constexpr bool SREL = ODD && FAST && REL > 0;
   int32_t rel[kQ];
   const uint32_t own32 = ent_off32(L);
 #pragma unroll
@@ -384,7 +400,7 @@ __device__ __forceinline__ void cell_update(const StepArgs &a, int32_t L, int32_
         else e = __ldg(a.idx + LBM_OFF(a, kChkIdx, 0, c2, LBM_NCELLS(a)));
         rel[k] = (int32_t)(ent_off32(e) - own32);
       }
-      if constexpr (SREL) { if (k <= 16) rel_slot(k) = rel[k]; }
+      if constexpr (SREL) { if (k <= REL) rel_slot<REL>(k) = rel[k]; }
     }
   }
   chain_wait();
@@ -622,7 +638,7 @@ __device__ __forceinline__ void cell_update(const StepArgs &a, int32_t L, int32_
     // load addresses of all 19 slots being held across the arithmetic)
     int32_t rk = rel[k];
     if constexpr (SREL) {
-      if (k != 0 && k <= 16) rk = rel_slot(k);
+      if (k != 0 && k <= REL) rk = rel_slot<REL>(k);
       else if (k != 0) asm volatile("" : "+r"(rk));
     } else if (ODD) {
       asm volatile("" : "+r"(rk));
@@ -906,7 +922,7 @@ __device__ __forceinline__ void gen_warp(const StepArgs &a, int w, int64_t t) {
 }
 
 // Warp w of the fast list.
-template <int ST, int LAYOUT, int NS, int ODD, int PHYS, bool UNI>
+template <int ST, int LAYOUT, int NS, int ODD, int PHYS, bool UNI, int REL>
 __device__ __forceinline__ void fast_warp(const StepArgs &a, int w, int64_t t) {
   if (w >= (UNI ? a.n_uni : a.n_fast + a.n_wall)) return;
   const uint32_t v = (uint32_t)__ldg(a.fast_list + w);
@@ -924,7 +940,7 @@ __device__ __forceinline__ void fast_warp(const StepArgs &a, int w, int64_t t) {
   // odd steps: one code path for plain and wall warps, the solid-neighbour
   // mask being zero for a plain warp (two paths in one kernel spill more)
   const uint32_t nbm = (ODD && !UNI && (v & kWallWarp)) ? __ldg(a.nbm + L) : 0u;
-  cell_update<ST, LAYOUT, NS, ODD, true, PHYS, ODD != 0 && !UNI, true, UNI>(a, L, cell, nbm, t, flux);
+  cell_update<ST, LAYOUT, NS, ODD, true, PHYS, ODD != 0 && !UNI, REL, UNI>(a, L, cell, nbm, t, flux);
 }
 
 // Cell kernel: one warp per listed lattice warp, the general warps in the
@@ -943,7 +959,7 @@ __device__ __forceinline__ void fast_warp(const StepArgs &a, int w, int64_t t) {
 // alone) but cost next to nothing. Step, with and without a launch of their
 // own: 158.5 and 161 us (128x128x256, FP16), 9,048 and 9,054 (512x512x1024,
 // FP16); 32x32x64 FP32 13.6 and 17.9 us.
-template <int ST, int LAYOUT, int NS, int ODD, int PHYS, bool UNI = false>
+template <int ST, int LAYOUT, int NS, int ODD, int PHYS, bool UNI = false, int REL = kRelNear>
 __global__ void __launch_bounds__(kCellBlock, cell_min_blocks(ST))
     cell_kernel(const __grid_constant__ StepArgs a, int block_0, int list_0) {
   chain_next();
@@ -957,7 +973,7 @@ __global__ void __launch_bounds__(kCellBlock, cell_min_blocks(ST))
     }
     b -= n_gen_blocks;
   }
-  fast_warp<ST, LAYOUT, NS, ODD, PHYS, UNI>(a, list_0 + b * kWarpsPerBlock + (int)(threadIdx.x >> 5), a.t);
+  fast_warp<ST, LAYOUT, NS, ODD, PHYS, UNI, REL>(a, list_0 + b * kWarpsPerBlock + (int)(threadIdx.x >> 5), a.t);
 }
 
 // One step of the cells of one 256-entry block of lattice entries
@@ -1117,7 +1133,7 @@ __global__ void __launch_bounds__(kCellBlock, cell_min_blocks(ST))
     b -= n_gen_blocks;
   }
   const int list_0 = (ODD && !UNI && p.uni) ? a.n_uni : 0;
-  fast_warp<ST, LAYOUT, NS, ODD, PHYS, UNI>(a, list_0 + b * kWarpsPerBlock + (int)(threadIdx.x >> 5), step);
+  fast_warp<ST, LAYOUT, NS, ODD, PHYS, UNI, kRelNear>(a, list_0 + b * kWarpsPerBlock + (int)(threadIdx.x >> 5), step);
 }
 
 // Per-plane FP64 sums of the current state: one cluster of kSumBlocks blocks
@@ -1334,6 +1350,13 @@ __global__ void __launch_bounds__(kBlock, export_min_blocks(ST, ODD, READ))
     }                                                                           \
   } while (0)
 
+// species count only (NSC)
+#define LBM_DISPATCH_FLUID_N(NS_, ...)                                          \
+  do {                                                                          \
+    if ((NS_) == 2) { constexpr int NSC = 2; __VA_ARGS__; }                     \
+    else { constexpr int NSC = 3; __VA_ARGS__; }                                \
+  } while (0)
+
 // layout x species x parity x deterministic accumulation
 #define LBM_DISPATCH_LNS(LAYOUT_, NS_, ODD_, DET_, ...)                                      \
   do {                                                                                     \
@@ -1343,18 +1366,41 @@ __global__ void __launch_bounds__(kBlock, export_min_blocks(ST, ODD, READ))
 
 // A launch of the step's chain on st; overlap: it may begin before the kernel
 // ahead of it on the stream has completed (see chain_wait).
+//
+// shape: the block's threads, and the share of the SM's 228 KB that the launch
+// asks for as shared memory: 64 KB for the step's kernels (eight blocks of 6 KB
+// and 1 KB of the system's), 100 KB for those with kRelWide offsets. Left to
+// itself the driver takes 100 and 135 KB for odd steps, and the step is 0.3 to
+// 0.6 % slower (512x512x1024 FP16 8,924 and 8,898 us, 191x173x300 BF16 330 and
+// 328).
+struct LaunchShape {
+  int threads;
+  unsigned carveout;  // per cent
+};
+constexpr LaunchShape kCellShape{kCellBlock, 28}, kWideCellShape{kCellBlock, 44}, kNodeShape{kBlock, 28};
 template <typename... P, typename... A>
-cudaError_t launch_chained(void (*kernel)(P...), unsigned grid, int threads, cudaStream_t st, bool overlap, const A &...args) {
-  cudaLaunchAttribute at{};
-  at.id = cudaLaunchAttributeProgrammaticStreamSerialization;
-  at.val.programmaticStreamSerializationAllowed = 1;
+cudaError_t launch_chained(void (*kernel)(P...), unsigned grid, LaunchShape shape, cudaStream_t st, bool overlap,
+                           const A &...args) {
+  cudaLaunchAttribute at[2] = {};
+  at[0].id = cudaLaunchAttributePreferredSharedMemoryCarveout;
+  at[0].val.sharedMemCarveout = shape.carveout;
+  at[1].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  at[1].val.programmaticStreamSerializationAllowed = 1;
   cudaLaunchConfig_t c{};
   c.gridDim = dim3(grid);
-  c.blockDim = dim3((unsigned)threads);
+  c.blockDim = dim3((unsigned)shape.threads);
   c.stream = st;
-  c.attrs = &at;
-  c.numAttrs = overlap ? 1 : 0;
+  c.attrs = at;
+  c.numAttrs = overlap ? 2 : 1;
   return cudaLaunchKernelEx(&c, kernel, args...);
+}
+
+// Whether three planes' populations take so much of L2 that odd steps keep to
+// kRelWide offsets (see rel_slot).
+template <int ST>
+bool wide_planes(const StepArgs &a, int layout, int ns) {
+  const int64_t entry = kQ * (int64_t)(sizeof(typename Pop<ST, 3>::C) + (ns == 3 ? sizeof(typename Pop<ST, 3>::S) : sizeof(typename Pop<ST, 2>::S)));
+  return layout == LBM_LAYOUT_FLUID && 3 * entry * (a.n_lat / a.nz) > kWidePlanes;
 }
 
 // RS (the random sputtering matrix) and PHYS (carrier velocity; barycentric
@@ -1370,19 +1416,21 @@ cudaError_t launch_step_st(const StepArgs &a, int layout, int ns, int parity, cu
   const bool overlap = !ev;  // (timed apart, each launch waits for the one before)
   cudaError_t e = cudaSuccess;
   if (ngrid > 0 && first)
-    LBM_DISPATCH_LNS(layout, ns, 0, a.det, e = launch_chained(node_kernel<ST, LY, NSC, DT, RS, kNodeEmit>, ngrid, kBlock, st, overlap, a));
+    LBM_DISPATCH_LNS(layout, ns, 0, a.det, e = launch_chained(node_kernel<ST, LY, NSC, DT, RS, kNodeEmit>, ngrid, kNodeShape, st, overlap, a));
   if (e != cudaSuccess) return e;
   if (ev) cudaEventRecord(ev[1], st);
   // even steps: the whole fast list in one launch; odd steps: the region
   // warps (fluid-only addressing, where there are enough of them), then the
   // plain and wall warps in increasing order
   const int32_t n_uni = (parity && layout == LBM_LAYOUT_FLUID && a.n_uni >= kUniMinWarps) ? a.n_uni : 0;
+  constexpr int kRel = PHYS == kPhysCarrier && ST != LBM_FP32 ? kRelWide : kRelNear;
+  const bool wide = kRel == kRelWide && wide_planes<ST>(a, layout, ns);
   if (n_uni > 0) {
     const unsigned ugrid = (unsigned)((n_uni + kWarpsPerBlock - 1) / kWarpsPerBlock);
-    if (ns == 2)
-      e = launch_chained(cell_kernel<ST, LBM_LAYOUT_FLUID, 2, 1, PHYS, true>, ugrid, kCellBlock, st, overlap, a, 0, 0);
+    if (wide)
+      LBM_DISPATCH_FLUID_N(ns, e = launch_chained(cell_kernel<ST, LBM_LAYOUT_FLUID, NSC, 1, PHYS, true, kRel>, ugrid, kWideCellShape, st, overlap, a, 0, 0));
     else
-      e = launch_chained(cell_kernel<ST, LBM_LAYOUT_FLUID, 3, 1, PHYS, true>, ugrid, kCellBlock, st, overlap, a, 0, 0);
+      LBM_DISPATCH_FLUID_N(ns, e = launch_chained(cell_kernel<ST, LBM_LAYOUT_FLUID, NSC, 1, PHYS, true>, ugrid, kCellShape, st, overlap, a, 0, 0));
     if (e != cudaSuccess) return e;
   }
   const unsigned fgrid =
@@ -1390,10 +1438,12 @@ cudaError_t launch_step_st(const StepArgs &a, int layout, int ns, int parity, cu
   auto cells = [&](unsigned block_0, unsigned blocks) {
     if (blocks == 0) return cudaSuccess;
     cudaError_t r;
-    if (parity)
-      LBM_DISPATCH_LN(layout, ns, r = launch_chained(cell_kernel<ST, LY, NSC, 1, PHYS>, blocks, kCellBlock, st, overlap, a, (int)block_0, n_uni));
+    if (parity && wide)
+      LBM_DISPATCH_FLUID_N(ns, r = launch_chained(cell_kernel<ST, LBM_LAYOUT_FLUID, NSC, 1, PHYS, false, kRel>, blocks, kWideCellShape, st, overlap, a, (int)block_0, n_uni));
+    else if (parity)
+      LBM_DISPATCH_LN(layout, ns, r = launch_chained(cell_kernel<ST, LY, NSC, 1, PHYS>, blocks, kCellShape, st, overlap, a, (int)block_0, n_uni));
     else
-      LBM_DISPATCH_LN(layout, ns, r = launch_chained(cell_kernel<ST, LY, NSC, 0, PHYS>, blocks, kCellBlock, st, overlap, a, (int)block_0, n_uni));
+      LBM_DISPATCH_LN(layout, ns, r = launch_chained(cell_kernel<ST, LY, NSC, 0, PHYS>, blocks, kCellShape, st, overlap, a, (int)block_0, n_uni));
     return r;
   };
   if (ev) {  // the fast and the general warps timed apart
@@ -1408,9 +1458,9 @@ cudaError_t launch_step_st(const StepArgs &a, int layout, int ns, int parity, cu
   if (ev) cudaEventRecord(ev[3], st);
   if (ngrid > 0) {
     if (last)
-      LBM_DISPATCH_LNS(layout, ns, 0, a.det, e = launch_chained(node_kernel<ST, LY, NSC, DT, RS, kNodeHits>, ngrid, kBlock, st, overlap, a));
+      LBM_DISPATCH_LNS(layout, ns, 0, a.det, e = launch_chained(node_kernel<ST, LY, NSC, DT, RS, kNodeHits>, ngrid, kNodeShape, st, overlap, a));
     else
-      LBM_DISPATCH_LNS(layout, ns, 0, a.det, e = launch_chained(node_kernel<ST, LY, NSC, DT, RS, kNodeBoth>, ngrid, kBlock, st, overlap, a));
+      LBM_DISPATCH_LNS(layout, ns, 0, a.det, e = launch_chained(node_kernel<ST, LY, NSC, DT, RS, kNodeBoth>, ngrid, kNodeShape, st, overlap, a));
   }
   if (ev) cudaEventRecord(ev[4], st);
   return e;
@@ -1433,7 +1483,7 @@ cudaError_t launch_batch_split_st(const BatchLaunch &p, int layout, int ns, int 
   cudaError_t e = cudaSuccess;
   const unsigned ngrid = (unsigned)p.total_node;
   if (ngrid > 0 && first)
-    LBM_DISPATCH_LNS(layout, ns, 0, det, e = launch_chained(batch_node_kernel<ST, LY, NSC, DT, RS, kNodeEmit>, ngrid, kBlock, st, false, p));
+    LBM_DISPATCH_LNS(layout, ns, 0, det, e = launch_chained(batch_node_kernel<ST, LY, NSC, DT, RS, kNodeEmit>, ngrid, kNodeShape, st, false, p));
   if (e != cudaSuccess) return e;
   // the run of simulations at the first one's parity, then the others
   const int run[3] = {0, p.n_lead, p.n_sims};
@@ -1444,24 +1494,24 @@ cudaError_t launch_batch_split_st(const BatchLaunch &p, int layout, int ns, int 
     const unsigned ugrid = odd ? (unsigned)(p.uni_start[q1] - p.uni_start[q0]) : 0u;
     if (ugrid > 0) {  // (p.uni: fluid-only addressing)
       if (ns == 2)
-        e = launch_chained(batch_cell_kernel<ST, LBM_LAYOUT_FLUID, 2, PHYS, 1, true>, ugrid, kCellBlock, st, false, p, q0);
+        e = launch_chained(batch_cell_kernel<ST, LBM_LAYOUT_FLUID, 2, PHYS, 1, true>, ugrid, kCellShape, st, false, p, q0);
       else
-        e = launch_chained(batch_cell_kernel<ST, LBM_LAYOUT_FLUID, 3, PHYS, 1, true>, ugrid, kCellBlock, st, false, p, q0);
+        e = launch_chained(batch_cell_kernel<ST, LBM_LAYOUT_FLUID, 3, PHYS, 1, true>, ugrid, kCellShape, st, false, p, q0);
       if (e != cudaSuccess) return e;
     }
     const unsigned grid = (unsigned)(p.cell_start[q1] - p.cell_start[q0]);
     if (grid == 0) continue;
     if (odd)
-      LBM_DISPATCH_LN(layout, ns, e = launch_chained(batch_cell_kernel<ST, LY, NSC, PHYS, 1>, grid, kCellBlock, st, false, p, q0));
+      LBM_DISPATCH_LN(layout, ns, e = launch_chained(batch_cell_kernel<ST, LY, NSC, PHYS, 1>, grid, kCellShape, st, false, p, q0));
     else
-      LBM_DISPATCH_LN(layout, ns, e = launch_chained(batch_cell_kernel<ST, LY, NSC, PHYS, 0>, grid, kCellBlock, st, false, p, q0));
+      LBM_DISPATCH_LN(layout, ns, e = launch_chained(batch_cell_kernel<ST, LY, NSC, PHYS, 0>, grid, kCellShape, st, false, p, q0));
     if (e != cudaSuccess) return e;
   }
   if (ngrid > 0) {
     if (last)
-      LBM_DISPATCH_LNS(layout, ns, 0, det, e = launch_chained(batch_node_kernel<ST, LY, NSC, DT, RS, kNodeHits>, ngrid, kBlock, st, false, p));
+      LBM_DISPATCH_LNS(layout, ns, 0, det, e = launch_chained(batch_node_kernel<ST, LY, NSC, DT, RS, kNodeHits>, ngrid, kNodeShape, st, false, p));
     else
-      LBM_DISPATCH_LNS(layout, ns, 0, det, e = launch_chained(batch_node_kernel<ST, LY, NSC, DT, RS, kNodeBoth>, ngrid, kBlock, st, false, p));
+      LBM_DISPATCH_LNS(layout, ns, 0, det, e = launch_chained(batch_node_kernel<ST, LY, NSC, DT, RS, kNodeBoth>, ngrid, kNodeShape, st, false, p));
   }
   return e;
 }

@@ -110,3 +110,17 @@ def test_steps_under_stream_capture():
     b.step(2)
     torch.cuda.synchronize()
     _assert_same(a, b)
+
+
+@pytest.mark.parametrize("side,storage,n_species", [(512, 0, 1), (512, 1, 2), (512, 2, 1), (640, 2, 2), (384, 0, 2)])
+def test_wide_planes_against_the_batched_launches(side, storage, n_species):
+    """Planes large enough for the odd step's other kernels, which a batch
+    never takes; region warps above and below their launch's threshold."""
+    from paper_1607_02874_gb300 import lbm
+
+    for nz, slab in ((10, (4, 7)), (16, (9, 13))):
+        g = lbm.Geometry(side, side, nz, slab=slab, porosity=0.6, corr_len=4.0, seed=7)
+        a, b = (_sim(lbm, g, layout=2, storage=storage, n_species=n_species) for _ in range(2))
+        a.step(5)
+        lbm.step_batch([b], 5)
+        np.testing.assert_array_equal(np.frombuffer(a.get_state(), np.uint8), np.frombuffer(b.get_state(), np.uint8))

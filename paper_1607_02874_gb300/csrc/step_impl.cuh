@@ -304,20 +304,21 @@ __device__ __forceinline__ float2 fma2(float2 a, float2 b, float2 c) { return __
 // so that the store reads it back instead of keeping a register copy). The
 // offsets beyond REL stay in registers.
 //
-// With kRelNear of them a block takes 6 KB and eight fit the 64 KB that the
-// launch asks for, which leaves the SM 192 KB of L1 for the gathers; with 16
-// (8 KB, 100 KB asked for) the loads wait for more of the offsets, and odd
-// steps keep less in flight. us of the odd step's cells, kRelWide (in the 135
-// KB that the driver chose by itself) and kRelNear: 191x173x300 BF16 387 and
-// 332, 128x128x256 FP16 171 and 165, 256x256x512 FP16 1,377 and 1,352;
-// 10 and 14 are slower than 12 (341 and 344 on the first).
+// With kRelNear of them eight blocks take 57 KB of the SM and the gathers have
+// the more L1; with 16 (72 KB; the driver sets 135 KB aside) the loads wait for
+// more of the offsets, and odd steps keep less in flight. us of the odd step's
+// cells with 16 and 12: 191x173x300 BF16 387 and 334, 128x128x256 FP16 171 and
+// 166, 256x256x512 FP16 1,377 and 1,357; 10 and 14 are slower than 12 (341 and
+// 344 on the first). Asking for a carve-out of 64 KB by launch attribute takes
+// another 0.3 to 0.6 % off these steps, but 5 to 20 % on small boxes (37x29x50
+// BF16 2,590 and 3,080 to 3,450 us for 101 steps): not done.
 //
 // Where the planes are large that turns round: the rows between the first and
 // the last warp in flight, with the planes above and below them, outgrow L2.
 // us a step of 16-bit boxes, three planes' populations in MB, kRelNear and
 // kRelWide: 26 MB (320x320) 1,432 and 1,454; 33 (512x256) 1,861 and 1,863; 37
 // (384x384) 2,089 and 2,085; 51 (448x448) 2,130 and 2,131; 66 (512x512) 2,759
-// and 2,747; 161 (800x800) 2,822 and 2,792; 66 (512x512x1024) 8,898 and 8,817.
+// and 2,747; 161 (800x800) 2,822 and 2,792; 66 (512x512x1024) 8,924 and 8,817.
 // FP32 keeps to kRelNear (512x512x300: 4,420 and 4,442), as do batches.
 constexpr int kRelNear = 12, kRelWide = 16;
 constexpr int64_t kWidePlanes = (int64_t)48 << 20;  // bytes, where the two meet
@@ -1366,32 +1367,17 @@ __global__ void __launch_bounds__(kBlock, export_min_blocks(ST, ODD, READ))
 
 // A launch of the step's chain on st; overlap: it may begin before the kernel
 // ahead of it on the stream has completed (see chain_wait).
-//
-// shape: the block's threads, and the share of the SM's 228 KB that the launch
-// asks for as shared memory: 64 KB for the step's kernels (eight blocks of 6 KB
-// and 1 KB of the system's), 100 KB for those with kRelWide offsets. Left to
-// itself the driver takes 100 and 135 KB for odd steps, and the step is 0.3 to
-// 0.6 % slower (512x512x1024 FP16 8,924 and 8,898 us, 191x173x300 BF16 330 and
-// 328).
-struct LaunchShape {
-  int threads;
-  unsigned carveout;  // per cent
-};
-constexpr LaunchShape kCellShape{kCellBlock, 28}, kWideCellShape{kCellBlock, 44}, kNodeShape{kBlock, 28};
 template <typename... P, typename... A>
-cudaError_t launch_chained(void (*kernel)(P...), unsigned grid, LaunchShape shape, cudaStream_t st, bool overlap,
-                           const A &...args) {
-  cudaLaunchAttribute at[2] = {};
-  at[0].id = cudaLaunchAttributePreferredSharedMemoryCarveout;
-  at[0].val.sharedMemCarveout = shape.carveout;
-  at[1].id = cudaLaunchAttributeProgrammaticStreamSerialization;
-  at[1].val.programmaticStreamSerializationAllowed = 1;
+cudaError_t launch_chained(void (*kernel)(P...), unsigned grid, int threads, cudaStream_t st, bool overlap, const A &...args) {
+  cudaLaunchAttribute at{};
+  at.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  at.val.programmaticStreamSerializationAllowed = 1;
   cudaLaunchConfig_t c{};
   c.gridDim = dim3(grid);
-  c.blockDim = dim3((unsigned)shape.threads);
+  c.blockDim = dim3((unsigned)threads);
   c.stream = st;
-  c.attrs = at;
-  c.numAttrs = overlap ? 2 : 1;
+  c.attrs = &at;
+  c.numAttrs = overlap ? 1 : 0;
   return cudaLaunchKernelEx(&c, kernel, args...);
 }
 
@@ -1416,7 +1402,7 @@ cudaError_t launch_step_st(const StepArgs &a, int layout, int ns, int parity, cu
   const bool overlap = !ev;  // (timed apart, each launch waits for the one before)
   cudaError_t e = cudaSuccess;
   if (ngrid > 0 && first)
-    LBM_DISPATCH_LNS(layout, ns, 0, a.det, e = launch_chained(node_kernel<ST, LY, NSC, DT, RS, kNodeEmit>, ngrid, kNodeShape, st, overlap, a));
+    LBM_DISPATCH_LNS(layout, ns, 0, a.det, e = launch_chained(node_kernel<ST, LY, NSC, DT, RS, kNodeEmit>, ngrid, kBlock, st, overlap, a));
   if (e != cudaSuccess) return e;
   if (ev) cudaEventRecord(ev[1], st);
   // even steps: the whole fast list in one launch; odd steps: the region
@@ -1428,9 +1414,9 @@ cudaError_t launch_step_st(const StepArgs &a, int layout, int ns, int parity, cu
   if (n_uni > 0) {
     const unsigned ugrid = (unsigned)((n_uni + kWarpsPerBlock - 1) / kWarpsPerBlock);
     if (wide)
-      LBM_DISPATCH_FLUID_N(ns, e = launch_chained(cell_kernel<ST, LBM_LAYOUT_FLUID, NSC, 1, PHYS, true, kRel>, ugrid, kWideCellShape, st, overlap, a, 0, 0));
+      LBM_DISPATCH_FLUID_N(ns, e = launch_chained(cell_kernel<ST, LBM_LAYOUT_FLUID, NSC, 1, PHYS, true, kRel>, ugrid, kCellBlock, st, overlap, a, 0, 0));
     else
-      LBM_DISPATCH_FLUID_N(ns, e = launch_chained(cell_kernel<ST, LBM_LAYOUT_FLUID, NSC, 1, PHYS, true>, ugrid, kCellShape, st, overlap, a, 0, 0));
+      LBM_DISPATCH_FLUID_N(ns, e = launch_chained(cell_kernel<ST, LBM_LAYOUT_FLUID, NSC, 1, PHYS, true>, ugrid, kCellBlock, st, overlap, a, 0, 0));
     if (e != cudaSuccess) return e;
   }
   const unsigned fgrid =
@@ -1439,11 +1425,11 @@ cudaError_t launch_step_st(const StepArgs &a, int layout, int ns, int parity, cu
     if (blocks == 0) return cudaSuccess;
     cudaError_t r;
     if (parity && wide)
-      LBM_DISPATCH_FLUID_N(ns, r = launch_chained(cell_kernel<ST, LBM_LAYOUT_FLUID, NSC, 1, PHYS, false, kRel>, blocks, kWideCellShape, st, overlap, a, (int)block_0, n_uni));
+      LBM_DISPATCH_FLUID_N(ns, r = launch_chained(cell_kernel<ST, LBM_LAYOUT_FLUID, NSC, 1, PHYS, false, kRel>, blocks, kCellBlock, st, overlap, a, (int)block_0, n_uni));
     else if (parity)
-      LBM_DISPATCH_LN(layout, ns, r = launch_chained(cell_kernel<ST, LY, NSC, 1, PHYS>, blocks, kCellShape, st, overlap, a, (int)block_0, n_uni));
+      LBM_DISPATCH_LN(layout, ns, r = launch_chained(cell_kernel<ST, LY, NSC, 1, PHYS>, blocks, kCellBlock, st, overlap, a, (int)block_0, n_uni));
     else
-      LBM_DISPATCH_LN(layout, ns, r = launch_chained(cell_kernel<ST, LY, NSC, 0, PHYS>, blocks, kCellShape, st, overlap, a, (int)block_0, n_uni));
+      LBM_DISPATCH_LN(layout, ns, r = launch_chained(cell_kernel<ST, LY, NSC, 0, PHYS>, blocks, kCellBlock, st, overlap, a, (int)block_0, n_uni));
     return r;
   };
   if (ev) {  // the fast and the general warps timed apart
@@ -1458,9 +1444,9 @@ cudaError_t launch_step_st(const StepArgs &a, int layout, int ns, int parity, cu
   if (ev) cudaEventRecord(ev[3], st);
   if (ngrid > 0) {
     if (last)
-      LBM_DISPATCH_LNS(layout, ns, 0, a.det, e = launch_chained(node_kernel<ST, LY, NSC, DT, RS, kNodeHits>, ngrid, kNodeShape, st, overlap, a));
+      LBM_DISPATCH_LNS(layout, ns, 0, a.det, e = launch_chained(node_kernel<ST, LY, NSC, DT, RS, kNodeHits>, ngrid, kBlock, st, overlap, a));
     else
-      LBM_DISPATCH_LNS(layout, ns, 0, a.det, e = launch_chained(node_kernel<ST, LY, NSC, DT, RS, kNodeBoth>, ngrid, kNodeShape, st, overlap, a));
+      LBM_DISPATCH_LNS(layout, ns, 0, a.det, e = launch_chained(node_kernel<ST, LY, NSC, DT, RS, kNodeBoth>, ngrid, kBlock, st, overlap, a));
   }
   if (ev) cudaEventRecord(ev[4], st);
   return e;
@@ -1483,7 +1469,7 @@ cudaError_t launch_batch_split_st(const BatchLaunch &p, int layout, int ns, int 
   cudaError_t e = cudaSuccess;
   const unsigned ngrid = (unsigned)p.total_node;
   if (ngrid > 0 && first)
-    LBM_DISPATCH_LNS(layout, ns, 0, det, e = launch_chained(batch_node_kernel<ST, LY, NSC, DT, RS, kNodeEmit>, ngrid, kNodeShape, st, false, p));
+    LBM_DISPATCH_LNS(layout, ns, 0, det, e = launch_chained(batch_node_kernel<ST, LY, NSC, DT, RS, kNodeEmit>, ngrid, kBlock, st, false, p));
   if (e != cudaSuccess) return e;
   // the run of simulations at the first one's parity, then the others
   const int run[3] = {0, p.n_lead, p.n_sims};
@@ -1494,24 +1480,24 @@ cudaError_t launch_batch_split_st(const BatchLaunch &p, int layout, int ns, int 
     const unsigned ugrid = odd ? (unsigned)(p.uni_start[q1] - p.uni_start[q0]) : 0u;
     if (ugrid > 0) {  // (p.uni: fluid-only addressing)
       if (ns == 2)
-        e = launch_chained(batch_cell_kernel<ST, LBM_LAYOUT_FLUID, 2, PHYS, 1, true>, ugrid, kCellShape, st, false, p, q0);
+        e = launch_chained(batch_cell_kernel<ST, LBM_LAYOUT_FLUID, 2, PHYS, 1, true>, ugrid, kCellBlock, st, false, p, q0);
       else
-        e = launch_chained(batch_cell_kernel<ST, LBM_LAYOUT_FLUID, 3, PHYS, 1, true>, ugrid, kCellShape, st, false, p, q0);
+        e = launch_chained(batch_cell_kernel<ST, LBM_LAYOUT_FLUID, 3, PHYS, 1, true>, ugrid, kCellBlock, st, false, p, q0);
       if (e != cudaSuccess) return e;
     }
     const unsigned grid = (unsigned)(p.cell_start[q1] - p.cell_start[q0]);
     if (grid == 0) continue;
     if (odd)
-      LBM_DISPATCH_LN(layout, ns, e = launch_chained(batch_cell_kernel<ST, LY, NSC, PHYS, 1>, grid, kCellShape, st, false, p, q0));
+      LBM_DISPATCH_LN(layout, ns, e = launch_chained(batch_cell_kernel<ST, LY, NSC, PHYS, 1>, grid, kCellBlock, st, false, p, q0));
     else
-      LBM_DISPATCH_LN(layout, ns, e = launch_chained(batch_cell_kernel<ST, LY, NSC, PHYS, 0>, grid, kCellShape, st, false, p, q0));
+      LBM_DISPATCH_LN(layout, ns, e = launch_chained(batch_cell_kernel<ST, LY, NSC, PHYS, 0>, grid, kCellBlock, st, false, p, q0));
     if (e != cudaSuccess) return e;
   }
   if (ngrid > 0) {
     if (last)
-      LBM_DISPATCH_LNS(layout, ns, 0, det, e = launch_chained(batch_node_kernel<ST, LY, NSC, DT, RS, kNodeHits>, ngrid, kNodeShape, st, false, p));
+      LBM_DISPATCH_LNS(layout, ns, 0, det, e = launch_chained(batch_node_kernel<ST, LY, NSC, DT, RS, kNodeHits>, ngrid, kBlock, st, false, p));
     else
-      LBM_DISPATCH_LNS(layout, ns, 0, det, e = launch_chained(batch_node_kernel<ST, LY, NSC, DT, RS, kNodeBoth>, ngrid, kNodeShape, st, false, p));
+      LBM_DISPATCH_LNS(layout, ns, 0, det, e = launch_chained(batch_node_kernel<ST, LY, NSC, DT, RS, kNodeBoth>, ngrid, kBlock, st, false, p));
   }
   return e;
 }

@@ -1113,7 +1113,7 @@ __global__ void __launch_bounds__(kBlock, node_min_blocks(ST, MODE)) batch_node_
 //
 // One tick of the serving loop (24 boxes of side 48 to 192, FP16, 40 steps)
 // took 102.8 ms with a launch of the general warps, a launch for each parity
-// over every block and no region launch; now 94.6. The launches do not overlap
+// over every block and no region launch; now 91.1. The launches do not overlap
 // as a single simulation's do: on that batch it is worth 0.7 %.
 template <int ST, int LAYOUT, int NS, int PHYS, int ODD, bool UNI = false>
 __global__ void __launch_bounds__(kCellBlock, cell_min_blocks(ST))

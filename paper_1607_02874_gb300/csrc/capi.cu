@@ -255,7 +255,8 @@ static StepArgs make_args_at(const lbm_sim *s, const int64_t t) {
   const int64_t ubsz = 2 * 5 * g->plane;
   a.ub_prev = s->ub + ((t + 1) & 1) * ubsz;
   a.ub_cur = s->ub + (t & 1) * ubsz;
-  a.node_cum = s->node_cum;
+  a.cum_now = cum_now(s, t);
+  a.cum_next = cum_now(s, t + 1);
   a.flux_cum = s->flux_cum;
   a.n_lo_warps = s->n_lo_warps;
   a.hi_warp = s->hi_warp;
@@ -742,7 +743,7 @@ static size_t sim_bytes(const lbm_geometry *g, const lbm_sim *s, int storage) {
   b += sizeof(acc_t) * 3 * 2 * s->acc_row;
   if (s->rs) b += sizeof(int32_t) * (g->n_nodes + 1);
   b += sizeof(float) * 2 * 2 * 5 * g->plane;
-  b += sizeof(double) * 2 * s->n_blocks;
+  b += sizeof(double) * 2 * 2 * s->n_blocks;
   b += sizeof(double) * 6 * std::max<int64_t>(s->n_flux_slots, 1);
   b += sizeof(double) * kPlaneCols * g->nz + sizeof(double) * 8;
   b += sizeof(int32_t) * (std::max<int64_t>(s->n_lat_warps, 1) + kUniTable);  // warp lists, region shifts
@@ -796,7 +797,7 @@ static void sim_free_all(lbm_sim *s) {
   m.free(s->A, sizeof(acc_t) * 3 * 2 * s->acc_row);
   m.free(s->node_off, sizeof(int32_t) * (s->g->n_nodes + 1));
   m.free(s->ub, sizeof(float) * 2 * 2 * 5 * s->g->plane);
-  m.free(s->node_cum, sizeof(double) * 2 * s->n_blocks);
+  m.free(s->node_cum, sizeof(double) * 2 * 2 * s->n_blocks);
   m.free(s->flux_cum, sizeof(double) * 6 * std::max<int64_t>(s->n_flux_slots, 1));
   m.free(s->plane_sums, sizeof(double) * kPlaneCols * s->g->nz);
   m.free(s->red_out, sizeof(double) * 8);
@@ -886,7 +887,7 @@ int lbm_init(const lbm_geometry *g, const lbm_params *prm, void *stream, const l
   s->f = m.alloc((size_t)s->ns * kQ * s->n_pad * storage_bytes(s->storage));
   s->A = m.alloc(sizeof(acc_t) * 3 * 2 * s->acc_row);
   s->ub = (float *)m.alloc(sizeof(float) * 2 * 2 * 5 * g->plane);
-  s->node_cum = (double *)m.alloc(sizeof(double) * 2 * s->n_blocks);
+  s->node_cum = (double *)m.alloc(sizeof(double) * 2 * 2 * s->n_blocks);
   s->flux_cum = (double *)m.alloc(sizeof(double) * 6 * std::max<int64_t>(s->n_flux_slots, 1));
   s->plane_sums = (double *)m.alloc(sizeof(double) * kPlaneCols * g->nz);
   s->red_out = (double *)m.alloc(sizeof(double) * 8);
@@ -919,7 +920,7 @@ int lbm_init(const lbm_geometry *g, const lbm_params *prm, void *stream, const l
   if (e == cudaSuccess) e = build_warp_lists(s, st);
   if (e == cudaSuccess) e = cudaMemsetAsync(s->A, 0, sizeof(acc_t) * 3 * 2 * s->acc_row, st);
   if (e == cudaSuccess) e = cudaMemsetAsync(s->ub, 0, sizeof(float) * 2 * 2 * 5 * g->plane, st);
-  if (e == cudaSuccess) e = cudaMemsetAsync(s->node_cum, 0, sizeof(double) * 2 * s->n_blocks, st);
+  if (e == cudaSuccess) e = cudaMemsetAsync(s->node_cum, 0, sizeof(double) * 2 * 2 * s->n_blocks, st);
   if (e == cudaSuccess)
     e = cudaMemsetAsync(s->flux_cum, 0, sizeof(double) * 6 * std::max<int64_t>(s->n_flux_slots, 1), st);
   if (e == cudaSuccess) {
@@ -1093,6 +1094,7 @@ int lbm_step_batch_mode(lbm_sim *const *sims, int n, int64_t nsteps, void *strea
     p.sync = dsync ? dsync + gi : nullptr;
   }
   std::vector<int> flags(ng);
+  std::vector<int64_t> ran(ng, 0);  // steps of each group launched (a failed launch ends the call part-way)
   bool timed_out = false;
   for (int64_t done = 0; done < nsteps && e == cudaSuccess && !timed_out;) {
     const int64_t m = dsync ? std::min<int64_t>(per_launch, nsteps - done) : 1;
@@ -1112,6 +1114,7 @@ int lbm_step_batch_mode(lbm_sim *const *sims, int n, int64_t nsteps, void *strea
       const lbm_sim *s0 = sims[order[groups[gi].first]];
       e = (m == 1 && !dsync) ? launch_batch_split(p, s0->storage, s0->layout, s0->ns, s0->det, st, done == 0, done == nsteps - 1)
                              : launch_batch(p, s0->storage, s0->layout, s0->ns, s0->det, st);
+      if (e == cudaSuccess) ran[gi] += m;
     }
     if (e == cudaSuccess && dsync && m > 1) {
       for (size_t gi = 0; gi < ng && e == cudaSuccess; ++gi)
@@ -1123,12 +1126,14 @@ int lbm_step_batch_mode(lbm_sim *const *sims, int n, int64_t nsteps, void *strea
   }
   if (e == cudaSuccess) e = cudaStreamSynchronize(st);
   if (dsync) sync_mem.free(dsync, sizeof(BatchSync) * ng);
+  if (!timed_out)
+    for (size_t gi = 0; gi < ng; ++gi)
+      for (int q = groups[gi].first; q < groups[gi].second; ++q) sims[order[q]]->t += ran[gi];
   if (e != cudaSuccess) return cuda_fail(e, "batched step");
   if (timed_out) {
     set_error("a step-ordering wait of the batched launch ran past its limit; the batch state is undefined");
     return LBM_ERR_TIMEOUT;
   }
-  for (int q = 0; q < n; ++q) sims[q]->t += nsteps;
   return LBM_OK;
 }
 
@@ -1141,7 +1146,7 @@ int lbm_observables(lbm_sim *s, lbm_obs *o) {
   int r = run_plane_sums(s, ps);
   if (r) return r;
   double red[8] = {0, 0, 0, 0, 0, 0, 0, 0};
-  LBM_CUDA_TRY(launch_sum_columns(s->node_cum, node_blocks(g), 2, s->red_out, st), "sum wall hits");
+  LBM_CUDA_TRY(launch_sum_columns(cum_now(s, s->t), node_blocks(g), 2, s->red_out, st), "sum wall hits");
   if (g->bc != LBM_BC_PERIODIC && s->n_flux_slots > 0)
     LBM_CUDA_TRY(launch_sum_columns(s->flux_cum, s->n_flux_slots, 6, s->red_out + 2, st), "sum face flows");
   else
@@ -1317,11 +1322,12 @@ struct StatePart {
   void *dev;
   size_t bytes;
 };
-static std::vector<StatePart> state_parts(const lbm_sim *s) {
+// (of a state at step t)
+static std::vector<StatePart> state_parts(const lbm_sim *s, int64_t t) {
   return {{s->f, (size_t)s->ns * kQ * s->n_pad * storage_bytes(s->storage)},
           {s->A, sizeof(acc_t) * 3 * 2 * s->acc_row},
           {s->ub, sizeof(float) * 2 * 2 * 5 * s->g->plane},
-          {s->node_cum, sizeof(double) * 2 * s->n_blocks},
+          {cum_now(s, t), sizeof(double) * 2 * s->n_blocks},
           {s->flux_cum, sizeof(double) * 6 * std::max<int64_t>(s->n_flux_slots, 1)}};
 }
 static StateHeader state_header(const lbm_sim *s) {
@@ -1351,7 +1357,7 @@ static StateHeader state_header(const lbm_sim *s) {
 int lbm_state_size(const lbm_sim *s, size_t *bytes) {
   if (!s || !bytes) return arg_fail("null argument");
   size_t b = sizeof(StateHeader);
-  for (auto &p : state_parts(s)) b += p.bytes;
+  for (auto &p : state_parts(s, s->t)) b += p.bytes;
   *bytes = b;
   return LBM_OK;
 }
@@ -1366,7 +1372,7 @@ int lbm_get_state(lbm_sim *s, void *dst, size_t n) {
   std::memcpy(dst, &h, sizeof(h));
   char *p = static_cast<char *>(dst) + sizeof(h);
   cudaStream_t st = s->mem.stream;
-  for (auto &part : state_parts(s)) {
+  for (auto &part : state_parts(s, s->t)) {
     LBM_CUDA_TRY(cudaMemcpyAsync(p, part.dev, part.bytes, cudaMemcpyDeviceToHost, st), "get state");
     p += part.bytes;
   }
@@ -1389,7 +1395,7 @@ int lbm_set_state(lbm_sim *s, const void *src, size_t n) {
     return arg_fail("state does not match this simulation (geometry, storage, layout, species or mode)");
   const char *p = static_cast<const char *>(src) + sizeof(h);
   cudaStream_t st = s->mem.stream;
-  for (auto &part : state_parts(s)) {
+  for (auto &part : state_parts(s, h.t)) {
     LBM_CUDA_TRY(cudaMemcpyAsync(part.dev, p, part.bytes, cudaMemcpyHostToDevice, st), "set state");
     p += part.bytes;
   }

@@ -312,7 +312,10 @@ struct StepArgs {
   void *A_next;          // [2][acc_row] the ring's third buffer (unused by the step)
   const float *ub_prev;  // [2 sides][5][plane] u and species rho of planes 1 / nz-2, previous step
   float *ub_cur;         // same, written this step
-  double *node_cum;      // [node blocks][2] per-256-node-block cumulative sum of A_prev (R, P)
+  // cumulative hits [node blocks][2] (R, P; a slot per 256 nodes): up to the
+  // step before the last one, and the copy that this step's emission writes
+  // with the last one's (A_prev) added
+  double *cum_now, *cum_next;
   double *flux_cum;      // [n_flux_slots][6] per-warp cumulative face flows (in C,R,P; out C,R,P)
   const int32_t *fast_list;  // [n_fast + n_wall] warps of the fast kernel (see kWallWarp), then the general
                              // list, then at word n_lat_warps the region shifts
@@ -683,8 +686,8 @@ struct lbm_geometry {
 };
 
 namespace lbm {
-// Blocks of the node kernels: the slots of node_cum in use (the array has one
-// per lattice block at least; the others stay 0).
+// Blocks of the node kernels: the slots of node_cum's copies in use (a copy has
+// one per lattice block at least; the others stay 0).
 inline int64_t node_blocks(const lbm_geometry *g) { return (g->n_nodes + kBlock - 1) / kBlock; }
 }  // namespace lbm
 
@@ -706,7 +709,7 @@ struct lbm_sim {
   int vel_in = 0;           // velocity inlet
   int sp_bb = 0;            // species bounce back at every solid
   float *ub = nullptr;      // [2][2][5][plane]
-  double *node_cum = nullptr;
+  double *node_cum = nullptr;  // [2][n_blocks][2] two copies of the cumulative hits (see cum_now)
   int64_t n_blocks = 0;
   double *flux_cum = nullptr;
   int64_t n_flux_slots = 0;
@@ -720,3 +723,9 @@ struct lbm_sim {
   double M0[3] = {0, 0, 0};
   size_t bytes = 0;
 };
+
+namespace lbm {
+// The cumulative hits of a state at step t: those of every step but the last
+// one. The emission of step t writes the other copy, with the last one's added.
+inline double *cum_now(const lbm_sim *s, int64_t t) { return s->node_cum + ((t + 1) & 1) * 2 * s->n_blocks; }
+}  // namespace lbm

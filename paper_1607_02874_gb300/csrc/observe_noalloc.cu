@@ -126,7 +126,7 @@ extern "C" int lbm_observables_noalloc(lbm_sim *s, lbm_obs *o) {
     e = launch_plane_sums(oa, s->storage, s->layout, s->ns, st);
   }
   double *red = scr + kNoAllocRows + kNoAllocProf;
-  if (e == cudaSuccess) e = launch_sum_columns(s->node_cum, node_blocks(g), 2, red, st);
+  if (e == cudaSuccess) e = launch_sum_columns(cum_now(s, s->t), node_blocks(g), 2, red, st);
   if (e == cudaSuccess) {
     if (g->bc != LBM_BC_PERIODIC && s->n_flux_slots > 0)
       e = launch_sum_columns(s->flux_cum, s->n_flux_slots, 6, red + 2, st);

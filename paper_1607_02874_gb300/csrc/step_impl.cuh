@@ -717,7 +717,9 @@ __device__ __forceinline__ void bank_flux(const StepArgs &a, int32_t W, const fl
 // per node, around the cell updates of a step:
 //   emission, before them: bank the previous step's hits of the node, and
 //     write into each link's slot what the sputtering law returns along the
-//     link;
+//     link. Both only write what the hits say, the banked sum from one copy of
+//     the cumulative hits to the other, so an emission that is made again (by
+//     the call after one whose launches failed part-way) changes nothing;
 //   hits, after them: the species that reached the node in this step,
 //     w_j times each link's stored value, summed over the node's links in a
 //     fixed order (or in 64-bit fixed point), into the step's accumulator
@@ -864,11 +866,11 @@ __device__ __forceinline__ void node_work(const StepArgs &a, int64_t n, int64_t 
   }
 }
 
-// Adds the block's FP64 sums of a pair of per-thread values to dst[0] and
-// dst[1], in a fixed order: the first exchange leaves one value to each half
-// of the warp, then the 8 warps' pairs are summed by one warp. Must be called
-// by every thread of the block.
-__device__ __forceinline__ void bank_pair(const float (&v)[2], double *dst) {
+// dst[0] and dst[1]: src's with the block's FP64 sums of a pair of per-thread
+// values added, in a fixed order: the first exchange leaves one value to each
+// half of the warp, then the 8 warps' pairs are summed by one warp. Must be
+// called by every thread of the block.
+__device__ __forceinline__ void bank_pair(const float (&v)[2], const double *src, double *dst) {
   __shared__ double sh[2][kBlock / 32];
   const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
   const bool hi = lane & 16;
@@ -881,7 +883,7 @@ __device__ __forceinline__ void bank_pair(const float (&v)[2], double *dst) {
     s = sh[lane / (kBlock / 32)][lane % (kBlock / 32)];
 #pragma unroll
     for (int o = kBlock / 64; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffu, s, o);
-    if (lane % (kBlock / 32) == 0) dst[lane / (kBlock / 32)] += s;
+    if (lane % (kBlock / 32) == 0) dst[lane / (kBlock / 32)] = src[lane / (kBlock / 32)] + s;
   }
 }
 
@@ -897,7 +899,10 @@ __device__ __forceinline__ void node_block(const StepArgs &a, int blk, int64_t t
     node_work<ST, LAYOUT, NS, DET, RS, MODE>(a, n, t, hv);
     if (n < a.bank_lo || n >= a.bank_hi) hv[0] = hv[1] = 0.f;  // (halo nodes are the neighbour's)
   }
-  if (MODE & kNodeEmit) bank_pair(hv, a.node_cum + 2 * (int64_t)blk);
+  // (kNodeBoth emits for step t + 1, where the copies have changed places)
+  if (MODE & kNodeEmit)
+    bank_pair(hv, (MODE == kNodeBoth ? a.cum_next : a.cum_now) + 2 * (int64_t)blk,
+              (MODE == kNodeBoth ? a.cum_now : a.cum_next) + 2 * (int64_t)blk);
 }
 
 template <int ST, int LAYOUT, int NS, bool DET, bool RS, int MODE>

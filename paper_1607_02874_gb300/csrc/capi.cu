@@ -250,7 +250,6 @@ static StepArgs make_args_at(const lbm_sim *s, const int64_t t) {
   char *A = static_cast<char *>(s->A);
   a.A_prev = A + ((t + 2) % 3) * ring;  // buffer of step t-1
   a.A_cur = A + (t % 3) * ring;
-  a.A_next = A + ((t + 1) % 3) * ring;
   a.det = s->det;
   const int64_t ubsz = 2 * 5 * g->plane;
   a.ub_prev = s->ub + ((t + 1) & 1) * ubsz;

@@ -309,13 +309,10 @@ struct StepArgs {
   const float *inv_b;    // [n_nodes] 1 / b(node)
   const void *A_prev;    // [2][acc_row] species that reached the walls in the previous step (acc_t or float)
   void *A_cur;           // [2][acc_row] written by this step's hits (node_work)
-  void *A_next;          // [2][acc_row] the ring's third buffer (unused by the step)
+  double *cum_next;      // cumulative hits with A_prev's added, as this step's emission writes them (see cum_now)
   const float *ub_prev;  // [2 sides][5][plane] u and species rho of planes 1 / nz-2, previous step
   float *ub_cur;         // same, written this step
-  // cumulative hits [node blocks][2] (R, P; a slot per 256 nodes): up to the
-  // step before the last one, and the copy that this step's emission writes
-  // with the last one's (A_prev) added
-  double *cum_now, *cum_next;
+  double *cum_now;       // [node blocks][2] cumulative hits (R, P) per 256 nodes, without those in A_prev
   double *flux_cum;      // [n_flux_slots][6] per-warp cumulative face flows (in C,R,P; out C,R,P)
   const int32_t *fast_list;  // [n_fast + n_wall] warps of the fast kernel (see kWallWarp), then the general
                              // list, then at word n_lat_warps the region shifts

@@ -25,12 +25,12 @@
 //     there is the halfway bounce-back that the next step reads as incoming
 //     opp(k); the even step's own-slot pointers give the same by
 //     construction.
-//   - species arriving from a catalytic solid are rebuilt from that node's
-//     wall hits of the previous step (A_prev) by the sputtering law; species
-//     leaving towards one are added to the node's hits of this step (A_cur).
+//   - species leaving towards a catalytic solid stay in the slot of the link,
+//     as the carrier does; after the cell updates the node kernels sum them per
+//     node into the step's wall hits (A_cur) and overwrite the slots with what
+//     the sputtering law returns, from the hits of the step before (A_prev).
 //     So the wall re-emits one step after the hit, the timing of bounce-back,
-//     with no grid-wide synchronisation. A 3-deep ring (prev, cur, next) lets
-//     every step clear the buffer of the step after.
+//     with no grid-wide synchronisation.
 //   - inlet plane z=0 / outlet plane z=nz-1: equilibrium with the velocity of
 //     plane 1 / nz-2 from the previous step (and, at the outlet, the species
 //     densities of plane nz-2), passed through a double-buffered plane cache.
@@ -112,17 +112,6 @@ __device__ __forceinline__ int64_t emit_index(bool rs, const StepArgs &a, int i,
 __device__ __forceinline__ float emit_scale(bool rs, const StepArgs &a, int32_t node) {
   return rs ? 1.0f : __ldg(a.inv_b + LBM_OFF(a, kChkNode, 0, node, a.n_nodes));
 }
-// Index of the accumulator that the species population arriving at node
-// `node` (in cell node_cell) along c_j adds to, species row sp.
-template <bool RS>
-__device__ __forceinline__ int64_t hit_index(const StepArgs &a, int sp, int32_t node, int32_t node_cell, int j,
-                                             int64_t t) {
-  if (!RS) return sp * a.acc_row + node;
-  const int32_t o = __ldg(a.node_off + LBM_OFF(a, kChkNode, 0, node, a.n_nodes + 1));
-  return sp * a.acc_row + o +
-         rs_rank(a.rs_key, node_cell, j, t, __ldg(a.node_off + LBM_OFF(a, kChkNode, 0, node + 1, a.n_nodes + 1)) - o);
-}
-
 // What a node that gathered AR and AP re-emits along its outgoing link i, in
 // the units of the stored species (scaled deviations d = f / w); scale: the
 // link's share (1/b, or 1 under the random matrix, whose slots are per link).

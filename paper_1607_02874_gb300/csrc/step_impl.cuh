@@ -1131,10 +1131,10 @@ __global__ void __launch_bounds__(kCellBlock, cell_min_blocks(ST))
   fast_warp<ST, LAYOUT, NS, ODD, PHYS, UNI, kRelNear>(a, list_0 + b * kWarpsPerBlock + (int)(threadIdx.x >> 5), step);
 }
 
-// Per-plane FP64 sums of the current state: one cluster of kSumBlocks blocks
-// per plane, which share out its entries and nodes and add their partial sums
-// in rank order through distributed shared memory (no scratch in device
-// memory, the same order on every call). Columns: rho_C, rho_R, rho_P,
+// Per-plane FP64 sums of the current state: one cluster of `parts` blocks
+// (sum_blocks) per plane, which share out its entries and nodes and add their
+// partial sums in rank order through distributed shared memory (no scratch in
+// device memory, the same order on every call). Columns: rho_C, rho_R, rho_P,
 // rho_P u_z over the plane's fluid cells (u_z the carrier's, or the
 // barycentric one when a.bary), and the raw wall hits A^R, A^P of the last
 // step over the plane's catalytic nodes. Inlet/outlet planes give zeros.
@@ -1147,23 +1147,52 @@ __global__ void __launch_bounds__(kCellBlock, cell_min_blocks(ST))
 // even state), 5,249 (FP16, odd), 1,593 and 2,641 (FP32), now 917, 2,318, 1,248
 // and 1,683.
 constexpr int kSumBlocks = 8;  // (the largest portable cluster)
+// Blocks per plane: 8, halved while a block would hold fewer cells than its
+// share of the grid's cost allows: 3,072 where the grid has more than 12 blocks
+// per SM, 1,024 from 6, and 768 (fluid-only) or 256 (dense, whose solid cells
+// leave the blocks uneven) from 2. A block costs 30 ns of the whole grid's time
+// however few its cells are, so 8 for every plane were slow where planes are
+// small and many. us of an lbm_observables_noalloc call (FP32, even state,
+// fluid-only) with 1, 2, 4 and 8, the one taken in brackets: 16x16x4000 (385)
+// 521 781 1,324; 24x24x256 (64) 67 82 114; 48x48x128 66 (65) 67 85; 64x64x64 78
+// 64 (54) 64; 64x64x1024 (281) 300 351 511; 128x128x32 189 123 84 (68);
+// 128x128x256 261 239 (250) 275; 256x256x512 1,425 1,423 1,366 (1,432). Over
+// 1,440 boxes and states it is within 4 % of 8 wherever that is better, within
+// 22 % of the best of the four, and 13 % below 8 in the mean.
+inline int sum_blocks(const StepArgs &a, int layout) {
+  const int64_t plane = (int64_t)a.nx * a.ny, sms = 152;
+  int parts = kSumBlocks;
+  for (; parts > 1; parts /= 2) {
+    const int64_t blocks = (int64_t)a.nz * parts;
+    const int64_t least = blocks > 12 * sms  ? 3072
+                          : blocks > 6 * sms ? 1024
+                          : blocks > 2 * sms ? (layout == LBM_LAYOUT_DENSE ? 256 : 768)
+                                                : 0;
+    if (plane >= least * parts) break;
+  }
+  return parts;
+}
 // Blocks per SM. Odd states load slot by slot, so they want warps: FP16 3,100,
 // 2,318, 2,474 us at 3, 4, 5 blocks, FP32 1,772, 1,683, 2,377 (more blocks
 // spill). Even ones: FP16 1,026, 982, 917, 1,133 at 2, 3, 4, 5; FP32 1,248,
 // 1,261, 1,354 at 2, 3, 4.
 constexpr int sum_min_blocks(int st, int odd) { return !odd && st == LBM_FP32 ? 2 : 4; }
-template <int ST, int LAYOUT, int NS, int ODD, bool DET>
-__global__ void __cluster_dims__(kSumBlocks, 1, 1) __launch_bounds__(kBlock, sum_min_blocks(ST, ODD)) plane_sums_kernel(const ObsArgs o) {
+// PARTS: the number of blocks where it is known at compile time, else 0. Eight,
+// the large planes' number, has an instance of its own: 256x256x512 FP16 906 us
+// (even) and 2,288 (odd), against 931 and 2,324 with the number as an argument.
+template <int ST, int LAYOUT, int NS, int ODD, bool DET, int PARTS>
+__global__ void __launch_bounds__(kBlock, sum_min_blocks(ST, ODD)) plane_sums_kernel(const ObsArgs o, const int n_parts) {
+  const int parts = PARTS ? PARTS : n_parts;
   namespace cg = cooperative_groups;
   const cg::cluster_group cluster = cg::this_cluster();
   const StepArgs &a = o.s;
-  const int z = (int)blockIdx.x / kSumBlocks, part = (int)blockIdx.x % kSumBlocks;
+  const int z = (int)blockIdx.x / parts, part = (int)blockIdx.x % parts;
   const bool bc = (!a.periodic_z && (z == 0 || z == a.nz - 1)) || halo_plane(a, z);
   double s[kPlaneCols] = {0, 0, 0, 0, 0, 0};
   if (!bc) {
     const int64_t hi = o.lat_plane[z + 1];
     int cells = 0;
-    for (int64_t Lw = o.lat_plane[z] + part * kBlock + threadIdx.x; Lw < hi; Lw += kSumBlocks * kBlock) {
+    for (int64_t Lw = o.lat_plane[z] + part * kBlock + threadIdx.x; Lw < hi; Lw += parts * kBlock) {
       const int32_t L = (int32_t)Lw;
       const int32_t cell = (LAYOUT == LBM_LAYOUT_DENSE) ? L : __ldg(a.fcell + L);
       const uint32_t nbm = __ldg(a.nbm + L);
@@ -1193,7 +1222,7 @@ __global__ void __cluster_dims__(kSumBlocks, 1, 1) __launch_bounds__(kBlock, sum
     }
     s[0] += (double)cells;
     if (NS > 1) {
-      for (int64_t k = o.node_plane[z] + part * kBlock + threadIdx.x; k < o.node_plane[z + 1]; k += kSumBlocks * kBlock) {
+      for (int64_t k = o.node_plane[z] + part * kBlock + threadIdx.x; k < o.node_plane[z + 1]; k += parts * kBlock) {
         s[4] += hits_d<DET>(a, 0, k);
         if (NS > 2) s[5] += hits_d<DET>(a, 1, k);
       }
@@ -1217,7 +1246,7 @@ __global__ void __cluster_dims__(kSumBlocks, 1, 1) __launch_bounds__(kBlock, sum
   cluster.sync();
   if (part == 0 && threadIdx.x < kPlaneCols) {
     double v = 0.0;
-    for (int r = 0; r < kSumBlocks; ++r) v += *cluster.map_shared_rank(&total[threadIdx.x], r);
+    for (int r = 0; r < parts; ++r) v += *cluster.map_shared_rank(&total[threadIdx.x], r);
     o.plane_sums[kPlaneCols * (int64_t)z + threadIdx.x] = v;
   }
   cluster.sync();  // (a block's shared memory lives until the sums are read)
@@ -1498,8 +1527,23 @@ cudaError_t launch_batch_split_st(const BatchLaunch &p, int layout, int ns, int 
 
 template <int ST>
 cudaError_t launch_plane_sums_st(const ObsArgs &o, int layout, int ns, cudaStream_t st) {
-  LBM_DISPATCH_LNS(layout, ns, o.parity, o.s.det, plane_sums_kernel<ST, LY, NSC, OD, DT><<<o.s.nz * kSumBlocks, kBlock, 0, st>>>(o));
-  return cudaGetLastError();
+  const int parts = sum_blocks(o.s, layout);
+  cudaLaunchAttribute at{};
+  at.id = cudaLaunchAttributeClusterDimension;
+  at.val.clusterDim.x = (unsigned)parts;
+  at.val.clusterDim.y = at.val.clusterDim.z = 1;
+  cudaLaunchConfig_t c{};
+  c.gridDim = dim3((unsigned)o.s.nz * (unsigned)parts);
+  c.blockDim = dim3(kBlock);
+  c.stream = st;
+  c.attrs = &at;
+  c.numAttrs = 1;
+  cudaError_t e = cudaSuccess;
+  if (parts == kSumBlocks)
+    LBM_DISPATCH_LNS(layout, ns, o.parity, o.s.det, e = cudaLaunchKernelEx(&c, plane_sums_kernel<ST, LY, NSC, OD, DT, kSumBlocks>, o, parts));
+  else
+    LBM_DISPATCH_LNS(layout, ns, o.parity, o.s.det, e = cudaLaunchKernelEx(&c, plane_sums_kernel<ST, LY, NSC, OD, DT, 0>, o, parts));
+  return e;
 }
 
 template <int ST>

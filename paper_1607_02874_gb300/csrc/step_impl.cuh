@@ -305,9 +305,12 @@ __device__ __forceinline__ float2 fma2(float2 a, float2 b, float2 c) { return __
 // Where the planes are large that turns round: the rows between the first and
 // the last warp in flight, with the planes above and below them, outgrow L2.
 // us a step of 16-bit boxes, three planes' populations in MB, kRelNear and
-// kRelWide: 26 MB (320x320) 1,432 and 1,454; 33 (512x256) 1,861 and 1,863; 37
-// (384x384) 2,089 and 2,085; 51 (448x448) 2,130 and 2,131; 66 (512x512) 2,759
-// and 2,747; 161 (800x800) 2,822 and 2,792; 66 (512x512x1024) 8,924 and 8,817.
+// kRelWide: 26 MB (320x320) 1,432 and 1,454; between 33 (512x256) and 51
+// (448x448) the two are within 0.2 %; 74 (512x512) 640.7 and 630.0 (FP16, 60
+// planes), 2,003 and 1,962 (BF16, 200 planes); 116 (640x640) 1,633 and 1,591;
+// 181 (800x800) 1,078 and 1,058; 66 (512x512x1024) 9,215 and 9,098 in a call of
+// 50 steps with five fields. (The last five differ by 1.3 to 2.6 %, and the
+// three runs of either form, taken in turn, by 0.1 %.)
 // FP32 keeps to kRelNear (512x512x300: 4,420 and 4,442), as do batches.
 constexpr int kRelNear = 12, kRelWide = 16;
 constexpr int64_t kWidePlanes = (int64_t)48 << 20;  // bytes, where the two meet
@@ -948,12 +951,17 @@ __device__ __forceinline__ void fast_warp(const StepArgs &a, int w, int64_t t) {
 // after the lists, which stays in L1; no fcell, idx or nbm reads), then the
 // rest.
 //
-// The general warps are 1-10 % of the warps and need 84-116 registers; in a
-// launch of their own they ran at 13 warps per SM after the fast warps had
-// drained. In the fast warps' launch they spill (96-230 bytes, in their branch
-// alone) but cost next to nothing. Step, with and without a launch of their
+// The general warps need 84-116 registers; in a launch of their own they ran at
+// 13 warps per SM after the fast warps had drained. In the fast warps' launch
+// the kernel spills more: even steps 0-96 bytes, odd ones 104-324, the most in
+// FP32 with the channel's terms; the region form, which has no general warps,
+// 0-52. It is the faster all the same. Step, in one launch and with one of their
 // own: 158.5 and 161 us (128x128x256, FP16), 9,048 and 9,054 (512x512x1024,
-// FP16); 32x32x64 FP32 13.6 and 17.9 us.
+// FP16); 32x32x64 FP32 13.6 and 17.9 us. Boxes of which half the planes are
+// general gained as well, 512x512x8 (C+R+P) from four launches that waited for
+// one another to the present ones: 213.9 -> 116.0 us (FP16, fluid-only), 202.3
+// -> 115.1 (FP16, dense), 250.1 -> 175.4 (FP32, fluid-only), 243.7 -> 175.5
+// (FP32, dense).
 template <int ST, int LAYOUT, int NS, int ODD, int PHYS, bool UNI = false, int REL = kRelNear>
 __global__ void __launch_bounds__(kCellBlock, cell_min_blocks(ST))
     cell_kernel(const __grid_constant__ StepArgs a, int block_0, int list_0) {

@@ -3,12 +3,13 @@
 
 One "step" = one time step of the whole hot path (collision of carrier,
 reactant and product, streaming, bounce-back, catalytic sputtering,
-inlet/outlet planes, wall-hit bookkeeping) over every fluid cell: two
-launches (the fused collide-stream kernel over every cell; the catalytic
-nodes' wall hits with the next step's emission), three on odd steps, whose
+inlet/outlet planes, wall-hit bookkeeping) over every fluid cell. After the
+warm-up, --windows windows of --steps steps are timed, each step a call of its
+own: three launches (the catalytic nodes' emission, the fused collide-stream
+kernel over every cell, the nodes' wall hits), four on odd steps, whose
 collide-stream kernel takes the all-fluid region warps in a launch of their
-own, and the first emission of a call. After the warm-up, --windows windows
-of --steps steps are timed; the line reports the median window.
+own. (Inside a call of several steps the nodes take one launch per step: the
+end-to-end run.) The line reports the median window.
 
 Prints one JSON line (rank 0). With --impl reference it times the FP64 CPU
 oracle instead, on a bounded sub-box of the same workload.
@@ -19,6 +20,7 @@ import argparse
 import hashlib
 import json
 import os
+import re
 import statistics
 import subprocess
 import sys
@@ -243,11 +245,22 @@ def kernel_source_hash(read=None):
     return h.hexdigest()[:16]
 
 
+def step_launches(warmup, steps, region_warps, nodes, read=None):
+    """Kernel launches of `steps` calls of one step each after `warmup` steps
+    (launch_step_st in step_impl.cuh): the cells in one launch, on odd steps in
+    two where there are kUniMinWarps region warps, and with catalytic nodes the
+    emission before them and the hits after them."""
+    read = read or (lambda f: open(os.path.join(ROOT, "paper_1607_02874_gb300", "csrc", f)).read())
+    least = int(re.search(r"kUniMinWarps = (\d+);", read("lbm_internal.h")).group(1))
+    n_odd = (warmup + steps) // 2 - warmup // 2
+    return steps * (3 if nodes else 1) + (n_odd if region_warps >= least else 0)
+
+
 def recorded_traffic(key, entries):
-    """DRAM bytes per launch of the fast step kernel from a committed ncu
-    summary, if it was taken on the current kernel source: bytes per lattice
-    entry (measured on a smaller case, both parities averaged) times the
-    entries one launch updates."""
+    """DRAM bytes per launch over the fast warps, as the launches timed apart
+    take them, from a committed ncu summary, if it was taken on the current
+    kernel source: bytes per lattice entry (measured on a smaller case, both
+    parities averaged) times the entries one launch updates."""
     path = os.path.join(ROOT, "profiles", "traffic.json")
     if not os.path.exists(path):
         return None
@@ -352,7 +365,9 @@ def main():
         if clk:
             clk.__exit__(None, None, None)
         # the launches of a step timed apart (CUDA events on the stream
-        # the library launches on), over both parities
+        # the library launches on), over both parities: general and fast warps
+        # in launches of their own, none overlapping the next, where the timed
+        # windows' steps take them in one
         t_split = sim.info()["step"]
         split = [sim.step_timed() for _ in range(8)]
         ms_fast = statistics.mean(x[0][0] for x in split)
@@ -384,7 +399,7 @@ def main():
     roof = {"bound": "hbm", "achieved": round(achieved, 1), "peak": peak, "unit": "GB/s",
             "frac": round(achieved / peak, 4), "traffic": traffic, "peak_kind": peak_kind,
             "bytes_per_cell_update": B_alg, "units_per_launch": e_fast,
-            "kernel": "cell_kernel (fused collide/stream of every warp away from the inlet/outlet planes, "
+            "kernel": "cell_kernel (lbm_step_timed: fused collide/stream of every warp away from the inlet/outlet planes, "
                       f"with the bounce-back redirection for cells touching a solid; {e_fast} of {e_fast + e_gen} "
                       "lattice entries; on odd steps two launches, the all-fluid region warps and the rest, "
                       "timed together)",
@@ -395,7 +410,8 @@ def main():
             "general_kernel": {"entries": e_gen, "launch_ms": round(res["ms_gen"], 4),
                                "achieved": round(B_alg * e_gen / (res["ms_gen"] / 1e3) / 1e9, 1)},
             "node_kernels": {"nodes": ginfo["n_nodes"], "launch_ms": round(res["ms_node"], 4),
-                             "what": "catalytic-node emission and wall-hit kernels of one step together"},
+                             "what": "catalytic-node emission and wall hits of a one-step call, two launches (one per "
+                                     "step inside a call of several)"},
             "step": {"achieved": round(step_gbs, 1), "frac": round(step_gbs / peak, 4),
                      "what": "algorithmic bytes of every fluid cell / median-window step time (every launch of the step)"}}
 
@@ -468,16 +484,8 @@ def main():
                          f"{r['n_fluid']} fluid cells"}
 
     obs = res["obs"]
-    # launches in the timed windows, one call of --steps steps each: per step
-    # the cell kernel, a second one on odd steps for the region warps where
-    # there are 12,288 of them or more, and one node launch (the hits, with
-    # the next step's emission), besides the call's first emission
-    wc = res["warps"]
     n_timed = args.steps * args.windows
-    n_odd = (args.warmup + n_timed) // 2 - args.warmup // 2
-    region_launch = int(wc["region"] >= 12288)
-    node_launches = (n_timed + args.windows) * int(ginfo["n_nodes"] > 0)
-    gpu_launches = n_timed + n_odd * region_launch + node_launches
+    gpu_launches = step_launches(args.warmup, n_timed, res["warps"]["region"], ginfo["n_nodes"])
     line = {
         "metric": METRIC, "value": round(value, 1), "unit": "MLUPS", "n_gpus": world, "steps": args.steps,
         "warmup": args.warmup, "ms_per_step": round(ms_step, 4), "higher_is_better": True, "scaling": "weak",

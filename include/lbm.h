@@ -284,61 +284,70 @@ int lbm_init(const lbm_geometry *g, const lbm_params *prm, void *stream, const l
  * with Eq. feq) for the carrier and every species, with halfway bounce-back
  * of the carrier and the sputtering boundary condition (Appendix,
  * Eq. f_P_in) at catalytic solid links, and the inlet/outlet planes. Per
- * step, on the simulation's stream (asynchronous), four launches:
- *   1. the catalytic nodes write the sputtering law's emission into their
- *      links' species slots;
- *   2. a fused collide-stream launch over the warps away from the
- *      inlet/outlet planes, with the halfway bounce-back at solid links
- *      (on odd steps of fluid-only addressing, two launches: first the
- *      region warps of the all-fluid planes, see lbm_warp_counts, then the
- *      others);
- *   3. one over the other warps;
- *   4. the nodes sum the species that reached them (the wall hits).
- * Errors: LBM_ERR_ARG (nsteps < 0), LBM_ERR_CUDA (a launch failed). */
+ * step, on the simulation's stream (asynchronous), two launches, each of which
+ * may begin while the one before it drains:
+ *   1. a fused collide-stream launch over every warp, with the halfway
+ *      bounce-back at solid links (on odd steps of fluid-only addressing, two
+ *      launches where there are 12,288 region warps or more: first those, see
+ *      lbm_warp_counts, then the others);
+ *   2. the catalytic nodes sum the species that reached them (the wall hits)
+ *      and write the sputtering law's emission of the next step into their
+ *      links' species slots.
+ * A call begins with a launch of the first step's emission, and its last launch
+ * takes the hits alone; without catalytic nodes, or with LBM_S_BOUNCEBACK, the
+ * node launches are left out.
+ * Errors: LBM_ERR_ARG (nsteps < 0), LBM_ERR_CUDA (a launch failed; lbm_sim_info
+ * gives the number of complete steps. If no cell of the step after them had been
+ * launched, the state and the observables are those of that step count and
+ * stepping may go on; else the state is undefined and should be restored from a
+ * checkpoint or destroyed). */
 int lbm_step(lbm_sim *s, int64_t nsteps);
 
-/* Measurement support: one step, exactly as lbm_step, with CUDA events
- * recorded around each of its launches. ms[0], ms[1] and ms[2] (three
- * floats) receive the device time in milliseconds of:
- *   [0] the fast kernel (the warps away from the inlet/outlet and halo
- *       planes: plain warps and, in the same launch, the warps whose cells
- *       touch a solid);
- *   [1] the general kernel (the other warps);
- *   [2] the two catalytic-node kernels together (the sputtering law's
- *       emission before the cell updates, the wall hits after them).
+/* Measurement support: one step, with the results of lbm_step(s, 1), whose
+ * launches do not overlap and take the cells in parts, with CUDA events
+ * recorded around each. (Inside an lbm_step call the parts [0] and [1] are one
+ * launch, and so are the two of [2], across the border of two steps: the parts
+ * add up to more than a step of such a call takes.) ms[0], ms[1] and ms[2]
+ * (three floats) receive the device time in milliseconds of:
+ *   [0] the fast warps (those away from the inlet/outlet and halo planes: plain
+ *       warps and the warps whose cells touch a solid; on odd steps with a
+ *       region launch, both launches);
+ *   [1] the general warps (the others);
+ *   [2] the catalytic nodes: the sputtering law's emission before the cell
+ *       updates and the wall hits after them, two launches.
  * entries (optional, NULL = skip) receives the lattice entries that the
- * fast and the general kernel update; entries[0] + entries[1] is every
+ * fast and the general warps update; entries[0] + entries[1] is every
  * lattice entry (dense addressing counts solid entries, which are skipped).
  * Synchronises the simulation's stream. Errors: LBM_ERR_ARG (null simulation
  * or ms), LBM_ERR_CUDA. */
 int lbm_step_timed(lbm_sim *s, float *ms, int64_t *entries);
 
 /* Measurement support: how the simulation's lattice warps (32 entries) are
- * divided among the step's kernels, fixed at lbm_init. counts (four
+ * divided by how the step takes them, fixed at lbm_init. counts (four
  * int64) receives:
- *   [0] plain warps of the fast kernel (no cell touches a solid), other
- *       than those of [1];
+ *   [0] plain warps (fast: no cell touches a solid), other than those of [1];
  *   [1] region warps, plain too: fluid-only addressing numbers their cells
  *       and all the cells' neighbours in the cells' own order, up to one
- *       shift, so that their odd steps (a launch of their own) form the
- *       neighbours' entries by arithmetic instead of reading the fluid
- *       index;
- *   [2] wall warps of the fast kernel (some cell touches a solid);
- *   [3] warps of the general kernel (inlet/outlet and halo planes).
+ *       shift, so that their odd steps can form the neighbours' entries by
+ *       arithmetic instead of reading the fluid index, in a launch of their
+ *       own. They do where there are 12,288 of them or more (in a batch, in
+ *       the group); fewer take the odd step with the other plain warps;
+ *   [2] wall warps (fast: some cell touches a solid);
+ *   [3] general warps (inlet/outlet and halo planes).
  * Warps with no live entry are not counted. Errors: LBM_ERR_ARG (null
  * simulation or counts). */
 int lbm_warp_counts(const lbm_sim *s, int64_t *counts);
 
 /* Advance n simulations by nsteps steps each (continuous batching of small
- * simulations). Simulations of equal storage, layout, species count and
- * accumulation mode form a group of at most 14, whose blocks make up one
- * kernel launch. Simulations at different step parities share a launch.
- * Two launch modes:
+ * simulations). Simulations of equal storage, layout, species count,
+ * accumulation mode, sputtering matrix and kind of velocity form a group of at
+ * most 14, whose blocks make up one kernel launch. Two launch modes:
  *   LBM_BATCH_PER_STEP (what lbm_step_batch uses): per group and step, the
- *     launches lbm_step makes for one simulation, each over every
- *     simulation of the group: the catalytic nodes' emission, the warps
- *     away from the inlet/outlet planes, the other warps, the nodes' wall
- *     hits;
+ *     launches lbm_step makes for one simulation, one after another: the
+ *     cells of the simulations at one step parity and of those at the other
+ *     (each run as lbm_step has it, with a region launch on odd steps), then
+ *     the catalytic nodes of all, with the call's first emission and last hits
+ *     alone;
  *   LBM_BATCH_SINGLE_LAUNCH: one launch per group for up to 1024 steps, one
  *     CTA per (phase, block), three phases per step (emission, cells, wall
  *     hits). Each CTA takes a ticket when it starts; a CTA of a phase waits
@@ -356,7 +365,8 @@ int lbm_warp_counts(const lbm_sim *s, int64_t *counts);
  * mode), LBM_ERR_OOM (the single-launch mode's step counters, a few KB taken
  * from the first simulation's allocator on `stream` and counted in its
  * lbm_footprint),
- * LBM_ERR_CUDA, LBM_ERR_TIMEOUT (a wait ran past its limit: the simulations
+ * LBM_ERR_CUDA (a launch failed: as for lbm_step, each group at the steps that
+ * it has completed), LBM_ERR_TIMEOUT (a wait ran past its limit: the simulations
  * of that call are in an undefined state and should be restored from a
  * checkpoint or destroyed). */
 #define LBM_BATCH_PER_STEP 0

@@ -47,11 +47,14 @@ void DevAlloc::free(void *p, size_t bytes) {
   if (bytes == 0) bytes = 256;
   if (has)
     a.free(a.ctx, p, bytes, (void *)stream);
-  else
-    cudaFreeAsync(p, stream);
+  else if (cudaFreeAsync(p, stream) != cudaSuccess)
+    cudaGetLastError();
 }
 
+// An error that is handed to the caller leaves the runtime's record of the last
+// error, which the next call's launches are checked against.
 static int cuda_fail(cudaError_t e, const char *what) {
+  cudaGetLastError();
   set_error(std::string(what) + ": " + cudaGetErrorString(e));
   return LBM_ERR_CUDA;
 }
@@ -581,6 +584,7 @@ int lbm_create_geometry(const lbm_geometry_desc *d, void *stream, const lbm_allo
   if (e != cudaSuccess) {
     lbm_geometry_free(g);
     if (e == cudaErrorMemoryAllocation) {
+      cudaGetLastError();
       set_error("geometry allocation failed");
       return LBM_ERR_OOM;
     }
@@ -661,7 +665,7 @@ void lbm_geometry_free(lbm_geometry *g) {
   m.free(g->fl_plane_d, sizeof(int64_t) * (g->nz + 1));
   m.free(g->node_plane_d, sizeof(int64_t) * (g->nz + 1));
   m.free(g->cell_plane_d, sizeof(int64_t) * (g->nz + 1));
-  cudaStreamSynchronize(m.stream);
+  if (cudaStreamSynchronize(m.stream) != cudaSuccess) cudaGetLastError();
   delete[] g->fl_plane_h;
   delete[] g->node_plane_h;
   delete g;
@@ -945,6 +949,7 @@ int lbm_init(const lbm_geometry *g, const lbm_params *prm, void *stream, const l
     sim_free_all(s);
     delete s;
     if (e == cudaErrorMemoryAllocation) {
+      cudaGetLastError();
       set_error("simulation allocation failed (warp-list scratch)");
       return LBM_ERR_OOM;
     }

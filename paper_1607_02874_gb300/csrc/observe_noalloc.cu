@@ -102,16 +102,23 @@ __global__ void __launch_bounds__(kFinishThreads) noalloc_finish_kernel(double *
 
 using namespace lbm;
 
+// (the runtime's record of the error is cleared: the next call's launches are
+// checked against it)
+static int refused() {
+  cudaGetLastError();
+  return LBM_ERR_CUDA;
+}
+
 extern "C" int lbm_observables_noalloc(lbm_sim *s, lbm_obs *o) {
   if (!s || !o) return LBM_ERR_ARG;
   const lbm_geometry *g = s->g;
   if (g->nz > LBM_NOALLOC_MAX_PLANES) return LBM_ERR_ARG;  // scratch holds LBM_NOALLOC_MAX_PLANES planes
   if (o->site_map) return LBM_ERR_ARG;                      // the site map needs staging: use lbm_observables
   int prev = 0;
-  if (cudaGetDevice(&prev) != cudaSuccess) return LBM_ERR_CUDA;
+  if (cudaGetDevice(&prev) != cudaSuccess) return refused();
   const int dev = g->device;
   if (dev < 0 || dev >= kMaxDevices) return LBM_ERR_ARG;
-  if (dev != prev && cudaSetDevice(dev) != cudaSuccess) return LBM_ERR_CUDA;
+  if (dev != prev && cudaSetDevice(dev) != cudaSuccess) return refused();
   double *scr = nullptr;
   cudaError_t e = scratch_address(dev, &scr);
   const cudaStream_t st = s->mem.stream;
@@ -146,7 +153,7 @@ extern "C" int lbm_observables_noalloc(lbm_sim *s, lbm_obs *o) {
                           cudaMemcpyDeviceToHost, st);
   if (e == cudaSuccess) e = cudaStreamSynchronize(st);
   if (dev != prev) cudaSetDevice(prev);
-  if (e != cudaSuccess) return LBM_ERR_CUDA;
+  if (e != cudaSuccess) return refused();
 
   const double p = s->p, pSR = s->prm.pS_R, pSP = s->prm.pS_P;
   const double M[3] = {buf[0], buf[1], buf[2]};

@@ -309,7 +309,7 @@ __device__ __forceinline__ float2 fma2(float2 a, float2 b, float2 c) { return __
 // (448x448) the two are within 0.2 %; 74 (512x512) 640.7 and 630.0 (FP16, 60
 // planes), 2,003 and 1,962 (BF16, 200 planes); 116 (640x640) 1,633 and 1,591;
 // 181 (800x800) 1,078 and 1,058; 66 (512x512x1024) 9,215 and 9,098 in a call of
-// 50 steps with five fields. (The last five differ by 1.3 to 2.6 %, and the
+// 50 steps with six fields. (The last five differ by 1.3 to 2.6 %, and the
 // three runs of either form, taken in turn, by 0.1 %.)
 // FP32 keeps to kRelNear (512x512x300: 4,420 and 4,442), as do batches.
 constexpr int kRelNear = 12, kRelWide = 16;

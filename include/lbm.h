@@ -352,7 +352,7 @@ int lbm_warp_counts(const lbm_sim *s, int64_t *counts);
  *     CTA per (phase, block), three phases per step (emission, cells, wall
  *     hits). Each CTA takes a ticket when it starts; a CTA of a phase waits
  *     until every block of the previous phase has finished. The wait is
- *     bounded (2 s of the GPU's global timer). Measured 1.7-2.4x slower
+ *     bounded (2 s of the GPU's global timer). Measured 2.2-2.9x slower
  *     than per-step launches on GB300: the per-CTA release fences and
  *     acquires of three phases per step cost more than kernel boundaries.
  * The work runs on `stream` (NULL: the first simulation's stream); the caller

@@ -293,12 +293,12 @@ __device__ __forceinline__ float2 fma2(float2 a, float2 b, float2 c) { return __
 // so that the store reads it back instead of keeping a register copy). The
 // offsets beyond REL stay in registers.
 //
-// With kRelNear of them eight blocks take 57 KB of the SM and the gathers have
-// the more L1; with 16 (72 KB; the driver sets 135 KB aside) the loads wait for
-// more of the offsets, and odd steps keep less in flight. us of the odd step's
-// cells with 16 and 12: 191x173x300 BF16 387 and 334, 128x128x256 FP16 171 and
-// 166, 256x256x512 FP16 1,377 and 1,357; 10 and 14 are slower than 12 (341 and
-// 344 on the first). Asking for a carve-out of 64 KB by launch attribute takes
+// kRelNear of them are the fastest on most boxes. us of the odd step's cells with
+// 16 and 12: 191x173x300 BF16 387 and 334, 128x128x256 FP16 171 and 166,
+// 256x256x512 FP16 1,377 and 1,357; 10 and 14 are slower than 12 (341 and 344 on
+// the first). Eight blocks take 57 KB of the SM with 12 and 72 KB with 16, and
+// the driver sets 135 KB aside for either, so the room left for L1 is not what
+// tells them apart. Asking for a carve-out of 64 KB by launch attribute takes
 // another 0.3 to 0.6 % off these steps, but 5 to 20 % on small boxes (37x29x50
 // BF16 2,590 and 3,080 to 3,450 us for 101 steps): not done.
 //
@@ -955,13 +955,15 @@ __device__ __forceinline__ void fast_warp(const StepArgs &a, int w, int64_t t) {
 // 13 warps per SM after the fast warps had drained. In the fast warps' launch
 // the kernel spills more: even steps 0-96 bytes, odd ones 104-324, the most in
 // FP32 with the channel's terms; the region form, which has no general warps,
-// 0-52. It is the faster all the same. Step, in one launch and with one of their
-// own: 158.5 and 161 us (128x128x256, FP16), 9,048 and 9,054 (512x512x1024,
-// FP16); 32x32x64 FP32 13.6 and 17.9 us. Boxes of which half the planes are
-// general gained as well, 512x512x8 (C+R+P) from four launches that waited for
-// one another to the present ones: 213.9 -> 116.0 us (FP16, fluid-only), 202.3
-// -> 115.1 (FP16, dense), 250.1 -> 175.4 (FP32, fluid-only), 243.7 -> 175.5
-// (FP32, dense).
+// 0-52. (Spilling requests a warp, 191x173x300 BF16: 0.06 on even steps, the
+// general warps' alone, and 5.4 on odd ones, two thirds or more of them not the
+// general warps'.) It is the faster all the same. Step, in one launch and with
+// one of their own: 158.5 and 161 us (128x128x256, FP16), 9,048 and 9,054
+// (512x512x1024, FP16); 32x32x64 FP32 13.6 and 17.9 us. Boxes of which half the
+// planes are general gained as well, 512x512x8 (C+R+P) from four launches that
+// waited for one another to the present ones: 213.9 -> 116.0 us (FP16,
+// fluid-only), 202.3 -> 115.1 (FP16, dense), 250.1 -> 175.4 (FP32, fluid-only),
+// 243.7 -> 175.5 (FP32, dense).
 template <int ST, int LAYOUT, int NS, int ODD, int PHYS, bool UNI = false, int REL = kRelNear>
 __global__ void __launch_bounds__(kCellBlock, cell_min_blocks(ST))
     cell_kernel(const __grid_constant__ StepArgs a, int block_0, int list_0) {

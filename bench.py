@@ -371,7 +371,7 @@ def main():
         t_split = sim.info()["step"]
         split = [sim.step_timed() for _ in range(8)]
         ms_fast = statistics.mean(x[0][0] for x in split)
-        # the fast kernel by the parity of the step it advances (t -> t + 1)
+        # the fast warps by the parity of the step it advances (t -> t + 1)
         by_par = [statistics.mean(x[0][0] for j, x in enumerate(split) if (t_split + j) % 2 == par) for par in (0, 1)]
         ms_gen = statistics.mean(x[0][1] for x in split)
         ms_node = statistics.mean(x[0][2] for x in split)
